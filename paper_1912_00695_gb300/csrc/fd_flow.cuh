@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R, YB) / W > 0 ? tma
             ok_all = false;  // a ring wait gave up (status set); the ring's phases are no longer known
             break;
         }
-        __syncthreads();  // the item's stores precede the flag
+        // (the segment ended with a CTA barrier: the item's stores precede the flag)
         if constexpr (EX) {
             if (s_ranges[3] > s_ranges[2]) {
                 flow_inject_extra(f, a, s, s_ranges[2], s_ranges[3], FORM == kExpanded);

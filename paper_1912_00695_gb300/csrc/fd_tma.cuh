@@ -98,6 +98,12 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
     return false;
 }
 
+// The same out of line, for the plane loop's rare wait that its first poll does not end:
+// the loop's code stays short (the polling inlined there cost 1 to 4 %).
+static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity) {
+    return mbar_wait_bounded(bar, parity);
+}
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar,
                                             int c0, int c1, int c2) {
     asm volatile(
@@ -260,7 +266,8 @@ __device__ __forceinline__ unsigned char *tma_ring_init(unsigned char *smem_raw)
 // of the shot described by `a` and `maps`. `g` counts the planes the CTA has
 // already streamed through its ring (it selects the stage and the mbarrier
 // phase, so consecutive segments share one ring without re-initialising it).
-// Returns false if a wait gave up (status set, copies in flight drained).
+// Returns false if a wait gave up (status set, copies in flight drained). Ends with a
+// CTA barrier, after every store of the segment.
 // COHERENT: u^n may have been written earlier in the same launch (the flow
 // schedule), so the queue prologue reads it through L2 instead of the
 // read-only path. step >= 0 replaces a.step (the flow schedule's steps share
@@ -405,7 +412,10 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
     // v - v is 0 for finite v and NaN otherwise, and NaN persists through the sum
     float2 nonfinite = f2(0.f, 0.f);
     bool over = acc.over;
-    bool failed = false;
+    // planes below issue_end are issued; 0 once this thread's wait has given up: it then waits
+    // no more, issues no more and runs on to the end of the segment (whose results are void:
+    // it returns false), so that the loop's barrier needs no vote
+    int issue_end = xe;
     int issued = min(S - 1, xe - xb);  // planes handed to the copy engine (tid 0's count)
     int it_failed = 0;                  // first plane whose wait gave up
     int stage = g0 % S;                 // ring stage and mbarrier phase of the current plane
@@ -414,28 +424,33 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
 #pragma unroll
     for (int r = 0; r < YB; ++r) any_own |= own[r];
 
+    // One CTA barrier per plane, without a vote; the copies are issued by warp 0 and the L2
+    // prefetches by warp 1, since the barrier makes the CTA as slow as its busiest warp.
+    // Against a voting barrier with everything issued by one thread (276^3, 200 steps of the
+    // flow in 32x16 tiles, one GB300): space order 4 / 8 / 12 / 16 factored 371.7 / 339.2 /
+    // 288.2 / 252.3 -> 373.4 / 351.1 / 302.1 / 259.2 Gpts/s, 8 expanded 269.9 -> 280.3, 12 in
+    // BF16 226.4 -> 239.6. The copies spread over all four warps gave 343 / 290 / 254 at 8 /
+    // 12 / 16; warps that run ahead of each other (full / empty mbarriers, or barrier.arrive
+    // by all but the issuing warp) 0.4x to 0.95x.
     for (int xo = xb; xo < xe; xo += U) {
 #pragma unroll
         for (int i = 0; i < U; ++i) {
             const int x = xo + i;
             if (x >= xe) break;
             const int it = x - xb;
-            const bool ok = mbar_wait_bounded(smem_addr(&bars[stage]), phase);
-            if (__syncthreads_or(!ok)) {
-                failed = true;
-                it_failed = it;
-                break;
-            }
-            if (tid == 0) {
-                if (x + S - 1 < xe) {
-                    // plane x + S - 1 takes the stage of plane x - 1, which every thread has
-                    // finished reading (it passed the barrier above)
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    issue(x + S - 1, stage == 0 ? S - 1 : stage - 1);
-                    ++issued;
+            if (!mbar_try_wait(smem_addr(&bars[stage]), phase))
+                if (issue_end > 0 && !mbar_wait_slow(smem_addr(&bars[stage]), phase)) {
+                    issue_end = 0;
+                    it_failed = it;
                 }
-                prefetch(x + 1 + kPrefetchAhead);
+            __syncthreads();  // every thread has finished reading the stage of plane x - 1
+            if (tid == 0 && x + S - 1 < issue_end) {
+                // plane x + S - 1 takes that stage
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                issue(x + S - 1, stage == 0 ? S - 1 : stage - 1);
+                ++issued;
             }
+            if (tid == 32) prefetch(x + 1 + kPrefetchAhead);
             const unsigned char *st = ring + stage * G::STAGE_BYTES;
 #pragma unroll
             for (int r = 0; r < YB; ++r)
@@ -685,16 +700,16 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
                 phase ^= 1u;
             }
         }
-        if (failed) break;
 #pragma unroll
         for (int r = 0; r < YB; ++r)
 #pragma unroll
             for (int k = 0; k < 2 * R; ++k) q[r][k] = q[r][k + U];
     }
-    if (failed) {
+    if (__syncthreads_or(issue_end == 0)) {
         // planes it_failed .. issued-1 are the only copies not yet waited for (one per stage)
         if (tid == 0) {
             if (a.status) atomicOr(a.status, kStatusTimeout);
+            if (issue_end > 0) it_failed = issued;  // this thread has waited for every copy it issued
             for (int it = it_failed; it < issued; ++it)
                 mbar_wait_bounded(smem_addr(&bars[(g0 + it) % S]), uint32_t((g0 + it) / S) & 1u);
         }
