@@ -566,11 +566,13 @@ int fd_slab_exchange(fd_handle *from, fd_handle *to, int level, void *stream);
  * of ld samples; q = 0 beyond ld), step n uses sample n (global step, from
  * step0). stream: a cudaStream_t (NULL = legacy default stream).
  *
- * Scratch: per-CTA maxima of |u| and the running maximum sit in one static
- * device array of 65,792 bytes (16,384 CTA slots + header) that every GPU
- * loading the library holds until exit. FD_EINVAL when one step would need
- * more than 16,384 CTAs (Ny*Nz above about 4.2 million points) or for bad
- * arguments; FD_ERANGE for a source outside the domain. The first call on a
+ * Scratch: the running maximum of |u| sits in one static device array of 256
+ * bytes that every GPU loading the library holds until exit. FD_EINVAL when a
+ * y-z plane holds more than 16,384 tiles of 8 x 32 points (Ny*Nz above about
+ * 4.2 million) or for bad arguments; FD_ERANGE for a source outside the domain.
+ * Rows and buffers of any float alignment are taken; where Nz is a multiple of 4
+ * and every buffer starts on 16 bytes (2 and 8 bytes) the inputs are copied in
+ * pieces of four (two) floats. The first call on a
  * device looks up that device's copy of the array (cudaGetSymbolAddress) and
  * its multiprocessor count (which sizes the x-chunks: four CTAs per
  * multiprocessor) once; make that first call before any stream capture. Every call on a device
