@@ -463,6 +463,12 @@ int autotune(fd_handle *hd) {
             if (xb >= 4 && xb < hd->Nx && std::find(v.begin(), v.end(), int(xb)) == v.end())
                 v.push_back(int(xb));
         }
+        // grids whose 8-plane chunks fit the slots at once: a step is one CTA's chain of planes,
+        // so shorter chunks shorten it (56^3, space order 4, one GB300: 2 planes 3.1 us a step,
+        // 12 planes 7.1; 84^3: 4 planes 5.3, 12 planes 7.9)
+        if (tiles * ((hd->Nx + 7) / 8) <= slots)
+            for (int xb : {2, 4, 8})
+                if (xb < hd->Nx && std::find(v.begin(), v.end(), xb) == v.end()) v.push_back(xb);
         return v;
     };
     auto take = [&](const TileShape &t, int xb) {
@@ -1682,6 +1688,17 @@ static int flow_tables(fd_handle *hd, int xb, int nbz, int nby, int nbx) {
 
 // Flow launch arguments for nt steps from the handle's state with x-chunks of
 // xb planes; *bytes: the zeroed prefix of the flow buffer (counter, abort, flags).
+// CTAs of the handle's flow kernel that the GPU holds at a time (0: no such kernel).
+static int flow_slots(fd_handle *hd, bool ex) {
+    int &flow_ctas = ex ? hd->flow_ctas_ex : hd->flow_ctas;
+    if (flow_ctas == 0) {
+        const int per_sm = tma_flow_ctas_per_sm(hd->r, hd->opt.form, hd->opt.storage, hd->tile_z, hd->tile_y,
+                                                hd->rows, ex);
+        if (per_sm > 0) flow_ctas = per_sm * device_sms();
+    }
+    return flow_ctas;
+}
+
 static int make_flow_args(fd_handle *hd, int nt, int xb, FlowArgs *f, size_t *bytes, int *ctas) {
     const int nbz = (hd->Nz + hd->tile_z - 1) / hd->tile_z, nby = (hd->Ny + hd->tile_y - 1) / hd->tile_y;
     const int nbx = (hd->Nx + xb - 1) / xb;
@@ -1703,16 +1720,8 @@ static int make_flow_args(fd_handle *hd, int nt, int xb, FlowArgs *f, size_t *by
     // the FP32 variant that samples receivers and adds extra sources per item
     const int ns = int(hd->sources.size()), n_x = ns > kFusedSources ? ns - kFusedSources : 0;
     const bool ex = hd->opt.storage == kF32 && (hd->n_rec > 0 || n_x > 0);
-    int &flow_ctas = ex ? hd->flow_ctas_ex : hd->flow_ctas;
-    if (flow_ctas == 0) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int per_sm = tma_flow_ctas_per_sm(hd->r, hd->opt.form, hd->opt.storage, hd->tile_z, hd->tile_y,
-                                                hd->rows, ex);
-        if (per_sm <= 0 || sms <= 0) return fail(FD_ENOTSUP, "no flow kernel for this launch shape");
-        flow_ctas = per_sm * sms;
-    }
+    const int flow_ctas = flow_slots(hd, ex);
+    if (flow_ctas == 0) return fail(FD_ENOTSUP, "no flow kernel for this launch shape");
     f->maps[0] = hd->tmaps[0];
     f->maps[1] = hd->tmaps[1];
     f->a[0] = make_args(hd, hd->step, 0);
@@ -1899,18 +1908,30 @@ static int flow_prepare(fd_handle *hd, int *nt) {
     // shorter x-chunks balance better and keep more items in flight on small grids,
     // longer ones claim fewer items and re-read fewer queue planes
     constexpr int kTuneSteps = 8, kLongSteps = 24;
+    // the x-chunk that gives about 1.7 items a step for each resident CTA: the items of a
+    // step then overlap the last step's tail, and no CTA carries a long chain of planes alone
+    const long long tiles = (long long)((hd->Nz + hd->tile_z - 1) / hd->tile_z) * ((hd->Ny + hd->tile_y - 1) / hd->tile_y);
+    const double even = double(hd->Nx) * double(tiles) / (1.7 * std::max(1, flow_slots(hd, hd->opt.storage == kF32 && extras != 0)));
     std::vector<int> cand;
-    for (int c : {8, 12, 16, 24, 32, 40, 48, 56, 64})
+    for (int c : {8, 12, 16, 24, 32, 40, 48, 56, even < 8.0 ? 4 : 64})
         if (c >= hd->r && c <= hd->Nx) cand.push_back(c);
     if (cand.empty()) cand.push_back(std::max(hd->r, 1));
     // warm-up + candidates, then the best length and the per-step launches each
     // timed afresh over kTuneSteps and kLongSteps
     const int needed = kTuneSteps * (int(cand.size()) + 1) + 2 * (kTuneSteps + kLongSteps);
     if (*nt < needed) {
-        // too few steps to time: the usual best for this call, the timing left to a
-        // later, longer call
-        hd->flow_wins = true;
-        return use(std::min(hd->Nx, std::max(40, hd->r)));
+        // too few steps to time: by rule for this call, the timing left to a later, longer
+        // call. The even x-chunk, in multiples of 4 planes up to 40 (measured best at 32x16
+        // tiles, space order 8: 150^3 8, 200^3 16, 276^3 40); below 6 planes the items' own
+        // start-up and flags weigh more than the launches and tails they save, and the
+        // per-step launches run instead. One GB300, 100 steps, us a step at space order 4 / 16:
+        // 56^3 3.1 / 4.4 per step against 6.5 / 12.5 flow at best (40-plane items 20 / 31),
+        // 84^3 5.3 / 7.5 against 5.0 / 13.3 (26 / 44), 150^3 12.2 / 21.2 against 11.9 / 17.3.
+        // Calls of fewer than 16 steps stay one flow launch: recording and instantiating
+        // their per-step graph would cost more than their steps.
+        hd->flow_wins = even >= 6.0 || *nt < 16;
+        const int xb = 4 * std::max(1, std::min(10, int(even / 4.0 + 0.5)));
+        return use(std::min(hd->Nx, std::max(xb, hd->r)));
     }
     float ms = 0.0f, best = 1e30f, flow_short = 0.0f, flow_long = 0.0f, step_short = 0.0f, step_long = 0.0f;
     int best_xb = cand[0];
