@@ -205,11 +205,14 @@ struct TmaShape {
     static constexpr int SMEM_BYTES = 128 + TmaPipe<R>::STAGES * STAGE_BYTES + 128;
 };
 
-// x-loop unroll (planes per queue shift): deeper unrolling saves queue moves but
-// grows the loop body; at R >= 5 the body of 2 planes measured fastest.
-template <int R, int FORM>
+// x-loop unroll (planes per queue shift). Deeper unrolling saves queue moves but grows the
+// loop body, and the four CTAs of an SM share its instruction cache. 276^3, Gpts/s at 4 / 2
+// / 1 planes: space order 4 373.3 / 373.4 / 372.0, in BF16 422.0 / 411.8 / 412.3; 8 361.4 /
+// 361.2 / 366.6, in FP16 291.0 / 295.9 / 287.1; 12 299.9 / 303.8 / 299.7; 16 267.2 / 268.3 /
+// 254.6; expanded 8 286.1 / 288.4 / 290.0, 16 172.6 / 184.6 / 165.7.
+template <int R, int FORM, typename T = float>
 struct TmaUnroll {
-    static constexpr int U = FORM == kFactored ? (R >= 5 ? 2 : 4) : 2;
+    static constexpr int U = FORM == kExpanded || R >= 5 ? 2 : R <= 2 ? 4 : Io<T>::kScaled ? 2 : 1;
 };
 
 // Sum of the two z taps at distance j of the pair of points (p, p+1) whose
@@ -262,6 +265,31 @@ __device__ __forceinline__ unsigned char *tma_ring_init(unsigned char *smem_raw)
     return ring;
 }
 
+// The fused sources among the points (x, y, z4 .. z4 + 3), added to their new values o: weight
+// w = f1 kd (factored; kd = 1 for FP32 storage) or dt^2 / r0 (expanded; f2 null where the damping
+// vanishes). Out of line: a tile has a source on one plane of one segment, and in the plane
+// loop the code (four sources for each unrolled plane) and its registers cost every plane:
+// 276^3, flow in 32x16 tiles, before -> after: space order 8 / 16 factored 351.1 / 259.2 ->
+// 361.4 / 268.3 Gpts/s, 8 expanded 280.3 -> 288.4, 4 in BF16 408 -> 422, 8 in FP16 (per-step
+// launches) 271 -> 291, 24 on 151 x 190 x 171 129.0 -> 143.5. (The same calls out of line
+// for the copies and prefetches, which run on every plane, cost 2 to 14 %; a copy of the
+// plane loop for undamped planes 1 to 12 %: the instruction cache is what both spend.)
+template <int FORM>
+static __device__ __noinline__ float4 tma_add_sources(const StepArgs &a, float4 o, int x, int y, int z4,
+                                                      long long step, const float *f1, const float *f2, float kd) {
+    for (int s = 0; s < a.ns && s < kFusedSources; ++s) {
+        const int p = a.sz[s] - z4;
+        if (a.sx[s] != x || a.sy[s] != y || p < 0 || p >= 4) continue;
+        const float qv = step >= 0 && step < a.ld ? __ldg(a.wavelet + (long long)s * a.ld + step) : 0.0f;
+        const float w = FORM == kFactored ? f1[p] * kd : a.dt2 * expanded_inv(fmaf(a.half_dt, f2 ? f2[p] : 0.0f, f1[p]));
+        if (p == 0) o.x = fmaf(w, qv, o.x);
+        if (p == 1) o.y = fmaf(w, qv, o.y);
+        if (p == 2) o.z = fmaf(w, qv, o.z);
+        if (p == 3) o.w = fmaf(w, qv, o.w);
+    }
+    return o;
+}
+
 // One segment of a CTA's work: planes [xb, xe) of tile (bz, by) of the y-z plane
 // of the shot described by `a` and `maps`. `g` counts the planes the CTA has
 // already streamed through its ring (it selects the stage and the mbarrier
@@ -285,7 +313,7 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
     using G = TmaShape<R, LZ, W, T, MODE == kModeAdjointGrad ? 2 : 0, YB>;
     using V = Vec4<T>;
     constexpr int RZ = G::RZ, LY = G::LY, TZ = G::TZ, TY = G::TY, SW = G::SW;
-    constexpr int U = TmaUnroll<R, FORM>::U;
+    constexpr int U = TmaUnroll<R, FORM, T>::U;
     constexpr int Q = 2 * R + U;  // queue slots: 2R planes of history/lookahead + U fronts
     constexpr int NWIN = 4 + 2 * RZ;  // z window values
     constexpr int S = TmaPipe<R>::STAGES;
@@ -327,7 +355,7 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
     // (the batch kernels) would otherwise be read again after every memory clobber of
     // the loop's barrier and copy code
     const int a_Nx = a.Nx, a_bx0 = a.bx0, a_bx1 = a.bx1;
-    const float a_half_dt = a.half_dt, a_dt2 = a.dt2;
+    const float a_half_dt = a.half_dt;
     // the row's points past its end (kept zero: the pitch padding)
     const unsigned tail_mask = (z4 + 1 >= a.Nz ? 2u : 0u) | (z4 + 2 >= a.Nz ? 4u : 0u) | (z4 + 3 >= a.Nz ? 8u : 0u);
     auto g_free = [&](int x) { return tile_yz_box && x >= a_bx0 && x < a_bx1; };
@@ -362,22 +390,17 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
         for (int d = 1; d <= kPrefetchAhead; ++d) prefetch(xb + d);
     }
 
-    // sources among each row's 4 points: bit s set, sub-index in src_p
-    unsigned src_mask[YB];
-    int src_p[YB][kFusedSources];
+    // planes of this segment where the tile has a fused source: [src_lo, src_hi] (empty
+    // for nearly every tile). The tile's planes there look the sources up in the arguments
+    // again: nothing per thread is kept for them.
+    int src_lo = xe, src_hi = -1;
 #pragma unroll
-    for (int r = 0; r < YB; ++r) {
-        src_mask[r] = 0;
-#pragma unroll
-        for (int s = 0; s < kFusedSources; ++s) {
-            src_p[r][s] = 0;
-            if (own[r] && s < a.ns && a.sy[s] == y0 + ty + r && a.sz[s] >= z4 && a.sz[s] < z4 + 4 &&
-                a.sx[s] >= xb && a.sx[s] < xe) {
-                src_mask[r] |= 1u << s;
-                src_p[r][s] = a.sz[s] - z4;
-            }
+    for (int s = 0; s < kFusedSources; ++s)
+        if (s < a.ns && a.sy[s] >= y0 && a.sy[s] < y0 + TY && a.sz[s] >= z0 && a.sz[s] < z0 + TZ && a.sx[s] >= xb &&
+            a.sx[s] < xe) {
+            src_lo = min(src_lo, a.sx[s]);
+            src_hi = max(src_hi, a.sx[s]);
         }
-    }
 
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     auto load_u = [&](int r, int x) -> float4 {
@@ -512,7 +535,6 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
                     cf2[r] = gf ? zero4
                                 : *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(st + G::OFF_F2) + po);
                 }
-                float sw[YB][4];
                 if constexpr (FORM == kFactored) {
                     // -6 u_c is added to each distance-j sum: exact zero for a constant field
                     float2 nsixA[YB], nsixB[YB];
@@ -564,10 +586,6 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
                             }
                             out[r] = make_float4(vA.x, vA.y, vB.x, vB.y);
                         }
-                        sw[r][0] = cf1[r].x * kd;  // kd = 1 for FP32 storage
-                        sw[r][1] = cf1[r].y * kd;
-                        sw[r][2] = cf1[r].z * kd;
-                        sw[r][3] = cf1[r].w * kd;
                     }
                 } else {
                     // expanded: every tap (u_tap - u_c) times (c_j dt^2/h^2)/r0
@@ -629,10 +647,6 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
                             vB = fma2(f2(1.0f - 2.0f * am[2], 1.0f - 2.0f * am[3]), hi2(cum[r]),
                                       fma2(f2(2.0f * am[2], 2.0f * am[3]), hi2(uc[r]), lapB[r]));
                         }
-                        if (src_mask[r]) {  // source weights dt^2 / r0, only where a source sits
-#pragma unroll
-                            for (int p = 0; p < 4; ++p) sw[r][p] = a_dt2 * inv[r][p];
-                        }
                         out[r] = make_float4(vA.x, vA.y, vB.x, vB.y);
                     }
                 }
@@ -640,20 +654,11 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
                 for (int r = 0; r < YB; ++r) {
                     if (!own[r]) continue;
                     float4 o = out[r];
-                    if (src_mask[r]) {
-#pragma unroll
-                        for (int s = 0; s < kFusedSources; ++s) {
-                            if (((src_mask[r] >> s) & 1u) && a.sx[s] == x) {
-                                const float qv = step < 0 ? source_value(a, s)
-                                                          : step < a.ld ? __ldg(a.wavelet + (long long)s * a.ld + step)
-                                                                        : 0.0f;
-                                const int p = src_p[r][s];
-                                if (p == 0) o.x = fmaf(sw[r][0], qv, o.x);
-                                if (p == 1) o.y = fmaf(sw[r][1], qv, o.y);
-                                if (p == 2) o.z = fmaf(sw[r][2], qv, o.z);
-                                if (p == 3) o.w = fmaf(sw[r][3], qv, o.w);
-                            }
-                        }
+                    if (x >= src_lo && x <= src_hi) {
+                        const int po = (ty + r) * TZ + 4 * lz;
+                        const float *w = reinterpret_cast<const float *>(st + G::OFF_F1) + po;
+                        o = tma_add_sources<FORM>(a, o, x, y0 + ty + r, z4, step < 0 ? a.step : step, w,
+                                                  gf ? nullptr : w + (G::OFF_F2 - G::OFF_F1) / 4, kd);
                     }
                     if (tail_mask) {  // row tail: keep the pitch padding zero
                         if (tail_mask & 2u) o.y = 0.f;
@@ -761,7 +766,7 @@ __device__ __forceinline__ void tma_sample_receivers(const StepArgs &a, float sc
 // share their halo rows in L2.
 template <int R, int FORM, int LZ, int W, typename T, int YB = 1>
 __global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R, YB) / W > 0 ? tma_warps_per_sm(R, YB) / W : 1))
-    fd_tma_kernel(const __grid_constant__ TmaMaps maps, const StepArgs a, int check) {
+    fd_tma_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ StepArgs a, int check) {
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     publish_scales<T>(a, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
     unsigned char *ring = tma_ring_init<R>(smem_dyn);
@@ -782,7 +787,7 @@ __global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R, YB) / W > 0 ? tma
 template <int R, int LZ, int W, int MODE>
 __global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R) / W > 0 ? tma_warps_per_sm(R) / W : 1)) fd_tma_grad_kernel(const __grid_constant__ TmaMaps maps,
                                                              const __grid_constant__ GradMaps gmaps,
-                                                             const StepArgs a, int check) {
+                                                             const __grid_constant__ StepArgs a, int check) {
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     unsigned char *ring = tma_ring_init<R>(smem_dyn);
     const ScaleState sc = read_scales<float>(a);
