@@ -64,6 +64,8 @@ std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int, int, int, int>, std::tuple<int, int, int, int>> g_tune_cache;
 // two-step kernel: (Nx, Ny, Nz, radius) -> x_block
 std::map<std::tuple<int, int, int, int>, int> g_tb_cache;
+// FWI gradient passes: (Nx, Ny, Nz, radius) -> x_block of the forward and of the adjoint pass
+std::map<std::tuple<int, int, int, int>, std::pair<int, int>> g_grad_cache;
 // flow schedule: (Nx, Ny, Nz, radius, form, tile_z, tile_y) -> (x_block, faster than per-step launches)
 std::map<std::tuple<int, int, int, int, int, int, int, int>, std::pair<int, bool>> g_flow_cache;
 
@@ -1107,17 +1109,27 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
     const int nseg = (nt + segment - 1) / segment;
     const bool ckpt = nseg > 1;
     const int tz = 32, ty = 16;  // the gradient passes' tile
-    const int xb = (hd->tile_z == tz && hd->tile_y == ty && hd->x_block > 0) ? hd->x_block
-                                                                              : heuristic_x_block(hd, tz, ty);
+    // x-chunk of each pass (0: not chosen yet)
+    const auto xb_key = std::make_tuple(hd->Nx, hd->Ny, hd->Nz, hd->r);
+    std::pair<int, int> xbs(0, 0);
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto it = g_grad_cache.find(xb_key);
+        if (it != g_grad_cache.end()) xbs = it->second;
+    }
     // workspace: the history of one segment (all steps without checkpoints), the
     // checkpoints, the gradient, two adjoint fields, the residuals, the receivers' node lists
     float *hist = nullptr, *ckp = nullptr, *grad = nullptr, *w[2] = {nullptr, nullptr}, *resid = nullptr;
     long long *node_off = nullptr;
     int *row = nullptr, *rec_idx = nullptr;
     float *rec_w = nullptr;
+    double *part = nullptr;  // partial sums of the misfit
+    cudaEvent_t tune_ev[2] = {nullptr, nullptr};
     auto release = [&]() {
-        void *bufs[] = {hist, ckp, grad, w[0], w[1], resid, node_off, row, rec_idx, rec_w};
+        void *bufs[] = {hist, ckp, grad, w[0], w[1], resid, node_off, row, rec_idx, rec_w, part};
         for (void *p : bufs) dev_free(p, st);
+        for (cudaEvent_t ev : tune_ev)
+            if (ev) cudaEventDestroy(ev);
     };
     // the receivers' spreading as a node-major list (fixed order within a node)
     struct Entry {
@@ -1158,7 +1170,8 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
         dev_alloc(reinterpret_cast<void **>(&node_off), h_node.size() * sizeof(long long), st) != cudaSuccess ||
         dev_alloc(reinterpret_cast<void **>(&row), h_row.size() * sizeof(int), st) != cudaSuccess ||
         dev_alloc(reinterpret_cast<void **>(&rec_idx), h_rec.size() * sizeof(int), st) != cudaSuccess ||
-        dev_alloc(reinterpret_cast<void **>(&rec_w), h_w.size() * sizeof(float), st) != cudaSuccess) {
+        dev_alloc(reinterpret_cast<void **>(&rec_w), h_w.size() * sizeof(float), st) != cudaSuccess ||
+        dev_alloc(reinterpret_cast<void **>(&part), kMisfitParts * sizeof(double), st) != cudaSuccess) {
         cudaGetLastError();
         release();
         return fail(FD_ENOMEM, "cannot allocate the gradient workspace (%d history levels, %d checkpoints)", segment,
@@ -1202,25 +1215,71 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
     }
     const bool check = check_enabled(hd);
     const int ns = int(hd->sources.size());
+    // `count` steps of a pass, launch(i, x_block) queueing step i. The first pass on a grid that
+    // is long enough times candidate x-chunks on two of its own steps each (any chunk gives
+    // the same bits): the shapes that fill the resident CTA slots best differ between the
+    // passes (the adjoint's ring holds two more tiles: three CTAs per SM instead of four) and
+    // from the plain step's. One GB300, space order 8, us a step of both passes with the
+    // plain step's chunk -> timed ones: 150^3 48.5 -> 41.8, 200^3 101.0 -> 90.6, 276^3 194.5 -> 192.2.
+    auto run_pass = [&](int count, int &chosen, auto &&launch) {
+        cudaError_t err = cudaSuccess;
+        const int fallback = heuristic_x_block(hd, tz, ty);
+        int i = 0;
+        if (chosen == 0) {
+            const long long tiles = (long long)((hd->Nz + tz - 1) / tz) * ((hd->Ny + ty - 1) / ty);
+            std::vector<int> cand = {fallback};  // (a warm-up: timed again below)
+            auto add = [&](long long c) {
+                if (c >= 1 && c <= hd->Nx && std::find(cand.begin() + 1, cand.end(), int(c)) == cand.end())
+                    cand.push_back(int(c));
+            };
+            for (int c : {12, 16, 20, 32, 64}) add(c);
+            for (int ctas : {3, 4, 6, 8}) {  // per SM: one and two waves
+                const long long chunks = (long long)ctas * device_sms() / tiles;
+                if (chunks >= 1) add((hd->Nx + chunks - 1) / chunks);
+            }
+            if (cand.size() == 1) cand.push_back(hd->Nx);
+            constexpr int kPer = 2;
+            if (count >= kPer * int(cand.size())) {
+                for (int k = 0; k < 2 && err == cudaSuccess; ++k)
+                    if (!tune_ev[k]) err = cudaEventCreate(&tune_ev[k]);
+                float best = 1e30f;
+                for (size_t c = 0; c < cand.size() && err == cudaSuccess; ++c) {
+                    err = cudaEventRecord(tune_ev[0], st);
+                    for (int k = 0; k < kPer && err == cudaSuccess; ++k) err = launch(i++, cand[c]);
+                    if (err == cudaSuccess) err = cudaEventRecord(tune_ev[1], st);
+                    if (err == cudaSuccess) err = cudaEventSynchronize(tune_ev[1]);
+                    float ms = 0.0f;
+                    if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, tune_ev[0], tune_ev[1]);
+                    if (c > 0 && err == cudaSuccess && ms < best) {
+                        best = ms;
+                        chosen = cand[c];
+                    }
+                }
+            }
+        }
+        const int xb = chosen > 0 ? chosen : fallback;
+        for (; i < count && err == cudaSuccess; ++i) err = launch(i, xb);
+        return err;
+    };
     // forward steps [n0, n1) from the handle's fields (cur), storing D^n at hist[n - n0]
     // (with_receivers: the traces of those steps are recorded)
     auto forward_d = [&](int n0, int n1, int &cur, bool with_receivers) {
-        cudaError_t err = cudaSuccess;
-        for (int n = n0; n < n1 && err == cudaSuccess; ++n) {
+        return run_pass(n1 - n0, xbs.first, [&](int i, int xb) {
+            const int n = n0 + i;
             StepArgs a = make_args(hd, n, cur);
             a.x_block = xb;
-            a.hist = hist + size_t(n - n0) * np;
+            a.hist = hist + size_t(i) * np;
             if (!with_receivers) {
                 a.n_rec = 0;
                 a.rec_sample = -1;
             }
-            err = launch_tma_grad_step(hd->r, kModeForwardD, fm[cur], gm, a, check, st);
+            cudaError_t err = launch_tma_grad_step(hd->r, kModeForwardD, fm[cur], gm, a, check, st);
             if (err == cudaSuccess && ns > kFusedSources)
                 err = launch_inject_extra(a, hd->d_src, hd->d_src + ns, hd->d_src + 2 * ns, kFusedSources,
                                           ns - kFusedSources, kF32, 0, hd->extra_distinct, st, a.hist);
             cur ^= 1;
-        }
-        return err;
+            return err;
+        });
     };
     int cur = hd->cur;
     e = cudaEventRecord(hd->ev0, st);  // device time of the passes: fd_last_forward_ms
@@ -1241,8 +1300,8 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
     }
     if (e == cudaSuccess) e = sample_level(hd, hd->ubuf[cur], nt, st);
     const int cur_end = cur;
-    // residual r = d - d_obs (in place over d_obs)
-    if (e == cudaSuccess) e = launch_residual(hd->d_traces, resid, size_t(nrec) * nt, st);
+    // residual r = d - d_obs (in place over d_obs) and the misfit's partial sums in FP64
+    if (e == cudaSuccess) e = launch_residual(hd->d_traces, resid, size_t(nrec) * nt, part, st);
     // adjoint pass, backward in time: w^k over w^{k+2} from w^{k+1}, the residual of
     // step k-1 injected at the receivers' nodes, gradient -= w^k D^{k-1}
     if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, fbytes, st);
@@ -1261,23 +1320,26 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
                 e = cudaMemcpyAsync(hd->ubuf[1], ckp + (slot + 1) * np, fbytes, cudaMemcpyDeviceToDevice, st);
             if (e == cudaSuccess) e = forward_d(n0, n1, rcur, false);
         }
-        for (int k = n1; k > n0 && e == cudaSuccess; --k) {
-            StepArgs a = make_args(hd, 0, 0);
-            a.u = w[c];
-            a.up = w[c ^ 1];
-            a.ns = 0;
-            a.n_rec = 0;
-            a.rec_sample = -1;
-            a.x_block = xb;
-            a.hist = hist + size_t(k - 1 - n0) * np;
-            a.hist_slot = k - 1 - n0;
-            a.grad = grad;
-            e = launch_tma_grad_step(hd->r, kModeAdjointGrad, am[c], gm, a, check, st);
-            if (e == cudaSuccess)
-                e = launch_adjoint_inject(w[c ^ 1], grad, a.hist, hd->f1, node_off, row, rec_idx, rec_w, resid, nt,
-                                          k - 1, inv_dt2, n_nodes, st);
-            c ^= 1;
-        }
+        if (e == cudaSuccess)
+            e = run_pass(n1 - n0, xbs.second, [&](int i, int xb) {
+                const int k = n1 - i;
+                StepArgs a = make_args(hd, 0, 0);
+                a.u = w[c];
+                a.up = w[c ^ 1];
+                a.ns = 0;
+                a.n_rec = 0;
+                a.rec_sample = -1;
+                a.x_block = xb;
+                a.hist = hist + size_t(k - 1 - n0) * np;
+                a.hist_slot = k - 1 - n0;
+                a.grad = grad;
+                cudaError_t err = launch_tma_grad_step(hd->r, kModeAdjointGrad, am[c], gm, a, check, st);
+                if (err == cudaSuccess)
+                    err = launch_adjoint_inject(w[c ^ 1], grad, a.hist, hd->f1, node_off, row, rec_idx, rec_w, resid,
+                                                nt, k - 1, inv_dt2, n_nodes, st);
+                c ^= 1;
+                return err;
+            });
     }
     if (e == cudaSuccess) e = cudaEventRecord(hd->ev1, st);
     hd->timed = e == cudaSuccess;
@@ -1301,10 +1363,11 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
         }
         hd->cur = rcur;
     }
-    // the traces (synthetic data) and the misfit (FP64 sum on the host)
-    std::vector<float> syn(size_t(nrec) * nt);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(syn.data(), hd->d_traces, syn.size() * sizeof(float), cudaMemcpyDeviceToHost, st);
+    // the traces (synthetic data), the misfit's partial sums and the gradient
+    double h_part[kMisfitParts];
+    if (e == cudaSuccess && syn_out)
+        e = cudaMemcpyAsync(syn_out, hd->d_traces, size_t(nrec) * nt * sizeof(float), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h_part, part, sizeof h_part, cudaMemcpyDeviceToHost, st);
     const size_t row_bytes = size_t(hd->Nz) * sizeof(float);
     if (e == cudaSuccess)
         e = cudaMemcpy2DAsync(grad_out, row_bytes, grad, size_t(hd->pz) * sizeof(float), row_bytes,
@@ -1312,12 +1375,14 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e);
     double J = 0.0;
-    for (size_t i = 0; i < syn.size(); ++i) {
-        const double d = double(syn[i]) - double(d_obs[i]);
-        J += 0.5 * d * d;
-    }
-    if (syn_out) std::memcpy(syn_out, syn.data(), syn.size() * sizeof(float));
+    for (double v : h_part) J += v;
     *misfit = J;
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto &known = g_grad_cache[xb_key];
+        if (xbs.first) known.first = xbs.first;
+        if (xbs.second) known.second = xbs.second;
+    }
     release();
     return check ? read_status(hd) : FD_OK;
 }

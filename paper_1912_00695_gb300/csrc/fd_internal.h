@@ -158,7 +158,8 @@ bool tma_box(int radius, int form, int storage, int tile_z, int tile_y, int rows
 cudaError_t launch_inject_extra(const StepArgs &a, const int *sx, const int *sy, const int *sz,
                                 int first, int count, int storage, int expanded, bool distinct, cudaStream_t s,
                                 float *hist = nullptr);
-cudaError_t launch_residual(const float *syn, float *obs_to_res, size_t n, cudaStream_t s);
+constexpr int kMisfitParts = 608;  // blocks of the residual kernel: partial sums of the misfit
+cudaError_t launch_residual(const float *syn, float *obs_to_res, size_t n, double *part, cudaStream_t s);
 cudaError_t launch_adjoint_inject(float *w, float *grad, const float *dhist, const float *f1,
                                   const long long *node_off, const int *row, const int *rec_idx, const float *rec_w,
                                   const float *resid, int nt, int t, float inv_dt2, int n_nodes, cudaStream_t s);

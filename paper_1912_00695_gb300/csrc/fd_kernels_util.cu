@@ -605,14 +605,28 @@ cudaError_t launch_adjoint_inject(float *w, float *grad, const float *dhist, con
     return counted(cudaGetLastError(), s);
 }
 
-__global__ void residual_kernel(const float *syn, float *obs_to_res, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        obs_to_res[i] = syn[i] - obs_to_res[i];
+// r = d - d_obs over d_obs, and each block's share of 1/2 sum (d - d_obs)^2 in FP64 (fixed grid
+// and tree: the same bits for the same data).
+__global__ void __launch_bounds__(256) residual_kernel(const float *syn, float *obs_to_res, long long n, double *part) {
+    __shared__ double sums[256];
+    double acc = 0.0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const float d = syn[i], o = obs_to_res[i];
+        const double diff = double(d) - double(o);
+        acc = fma(0.5 * diff, diff, acc);
+        obs_to_res[i] = d - o;
+    }
+    sums[threadIdx.x] = acc;
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if (threadIdx.x < h) sums[threadIdx.x] += sums[threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) part[blockIdx.x] = sums[0];
 }
 
-cudaError_t launch_residual(const float *syn, float *obs_to_res, size_t n, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    residual_kernel<<<608, 256, 0, s>>>(syn, obs_to_res, (long long)n);
+cudaError_t launch_residual(const float *syn, float *obs_to_res, size_t n, double *part, cudaStream_t s) {
+    residual_kernel<<<kMisfitParts, 256, 0, s>>>(syn, obs_to_res, (long long)n, part);
     return counted(cudaGetLastError(), s);
 }
 
