@@ -456,7 +456,7 @@ int autotune(fd_handle *hd) {
             return v;
         }
         const long long warps = (long long)tz * ty / (128 * rows);  // 4 points per thread and row
-        const long long slots = (long long)sms * std::max(1LL, tma_warps_per_sm(hd->r, rows) / warps);
+        const long long slots = (long long)sms * std::max(1LL, tma_warps_per_sm(hd->r, rows, hd->opt.form) / warps);
         const long long tiles = (long long)((hd->Nz + tz - 1) / tz) * ((hd->Ny + ty - 1) / ty);
         for (int waves = 1; waves <= 3; ++waves) {
             const long long chunks = slots * waves / tiles;  // chunks per tile that still fit

@@ -168,7 +168,7 @@ static __device__ __noinline__ void flow_region_ranges(const FlowArgs &f, int re
 // EX: the FP32 variant with receivers and extra sources handled per item; the
 // plain variant carries none of that code.
 template <int R, int FORM, int LZ, int W, int YB = 1, typename T = float, bool EX = false>
-__global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R, YB) / W > 0 ? tma_warps_per_sm(R, YB) / W : 1))
+__global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R, YB, FORM) / W > 0 ? tma_warps_per_sm(R, YB, FORM) / W : 1))
     fd_tma_flow_kernel(const __grid_constant__ FlowArgs f, int check) {
     static_assert(std::is_same<T, float>::value || std::is_same<T, __nv_bfloat16>::value,
                   "the flow schedule stores FP32 or BF16 (FP16 needs per-level scales)");

@@ -765,7 +765,7 @@ __device__ __forceinline__ void tma_sample_receivers(const StepArgs &a, float sc
 // CTAs resident at any moment cover neighbouring tiles at the same planes and
 // share their halo rows in L2.
 template <int R, int FORM, int LZ, int W, typename T, int YB = 1>
-__global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R, YB) / W > 0 ? tma_warps_per_sm(R, YB) / W : 1))
+__global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R, YB, FORM) / W > 0 ? tma_warps_per_sm(R, YB, FORM) / W : 1))
     fd_tma_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ StepArgs a, int check) {
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     publish_scales<T>(a, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
