@@ -8,11 +8,12 @@
 // planes extended by R on both sides, at step-1 plane x every thread
 //  * computes u^{n+1}(x) at its 4 points of E from u^n (register queue for the
 //    x taps, the TMA-fed halo box for y and z, exactly the single-step
-//    kernel's per-point arithmetic) and puts it in a shared ring of 2R+1
+//    kernel's per-point arithmetic) and puts it in a shared ring of
 //    u^{n+1} planes (zero outside the domain: the Dirichlet halo of u^{n+1});
 //    points of T inside [xb, xe) are also stored to global memory (u^{n+1});
 //  * after a CTA barrier, computes u^{n+2}(x - R) at its points of T from the
-//    u^{n+1} ring (x, y and z taps), u^n(x - R) (the oldest queue entry), and
+//    u^{n+1} ring (y and z taps; the x taps are the thread's own results, at R = 1
+//    kept in registers), u^n(x - R) (the oldest queue entry), and
 //    w, g of plane x - R (a register queue of R+1 planes), and stores it.
 // Per pair of steps HBM sees u^n, u^{n-1}, w (g in the layer) read and
 // u^{n+1}, u^{n+2} written: 20 B per point (plus g in the layer) instead of 32
@@ -21,6 +22,12 @@
 // buffers: u^{n+1} cannot overwrite u^{n-1}, which overlapping CTAs still read.
 // Sources of both steps are fused; receivers and the other storages are not
 // supported here.
+// Bound: latency at 16 warps per SM (two CTAs; shared memory and registers allow no third)
+// and two CTA barriers per plane, well above the HBM time of its 10.4 B per point and
+// step. The barriers carry no vote, the sources sit out of line, the L2 prefetches are
+// issued by a second warp, and four stages are in flight: 276^3, space order 2, 300 steps,
+// one GB300 407 -> 463 Gpts/s (three stages and ring x taps: 442); 84^3 115 -> 144;
+// 343 x 220 x 350 385 -> 460.
 #pragma once
 
 #include "fd_tma.cuh"
@@ -42,8 +49,12 @@ struct Tb2Shape {
     static constexpr int OFF_FRONT = HALO, OFF_UP = HALO + PT_RAW, OFF_F1 = HALO + 2 * PT_RAW,
                          OFF_F2 = HALO + 3 * PT_RAW;
     static constexpr int STAGE_BYTES = HALO + 4 * PT_RAW;
-    static constexpr int STAGES = 3;
-    static constexpr int NU1 = 2 * R + 1;  // u^{n+1} planes the second step reads
+    static constexpr int STAGES = 4;
+    // The second step's x taps are the thread's own earlier results: at R = 1 they stay in
+    // registers and the ring holds the planes that the y and z taps still read (at R = 2 the
+    // registers are worth more: 359.7 against 355.9 Gpts/s at 276^3, space order 4)
+    static constexpr bool OWN_X = R == 1;
+    static constexpr int NU1 = OWN_X ? R + 1 : 2 * R + 1;  // u^{n+1} planes in the ring
     static constexpr int U1_OFF = STAGES * STAGE_BYTES;
     static constexpr int BAR_OFF = U1_OFF + NU1 * PT_RAW;
     static constexpr int SMEM_BYTES = BAR_OFF + 64 + 128;
@@ -80,15 +91,11 @@ __device__ __forceinline__ float4 tb2_update(const float *rowp, const float *win
     return make_float4(vA.x, vA.y, vB.x, vB.y);
 }
 
-__device__ __forceinline__ float tb2_source(const StepArgs &a, int s, long long step) {
-    return (step >= 0 && step < a.ld) ? __ldg(a.wavelet + (long long)s * a.ld + step) : 0.0f;
-}
-
 // u^{n+1} into out1 and u^{n+2} into out2 from u^n = a.u, u^{n-1} = a.up (read
 // through `maps`), global step n = a.step. CTA (bz, by, bx): T origin
 // (bz*56, by*(16-2R)), planes [bx x_block, (bx+1) x_block).
 template <int R>
-__global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__ TmaMaps maps, const StepArgs a,
+__global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ StepArgs a,
                                                           float *out1, float *out2, int check) {
     using G = Tb2Shape<R>;
     constexpr int S = G::STAGES, U = G::U, Q = 2 * R + U, NWIN = 4 + 2 * G::HZ, EZ = G::EZ, SW = G::SW;
@@ -132,21 +139,27 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
         tma_load_3d(smem_addr(st + G::OFF_F1), &maps.f1_pt, bar, ze0, ye0, x);
         if (need_g) tma_load_3d(smem_addr(st + G::OFF_F2), &maps.f2_pt, bar, ze0, ye0, x);
     };
+    // the same boxes of plane x into L2, further ahead
+    auto prefetch = [&](int x) {
+        if (x < xend) {
+            tma_prefetch_3d(&maps.up_pt, ze0, ye0, x);
+            tma_prefetch_3d(&maps.f1_pt, ze0, ye0, x);
+            if (!g_free(x)) tma_prefetch_3d(&maps.f2_pt, ze0, ye0, x);
+            if (x + R < a.Nx) tma_prefetch_3d(&maps.u_pt, ze0, ye0, x + R);
+        }
+    };
     const int n_planes = xend - xs;
     if (tid == 0)
         for (int s = 0; s < S - 1 && s < n_planes; ++s) issue(xs + s, s);
 
-    // sources at this thread's 4 points of E: bit s set, sub-index in src_p
-    unsigned src_mask = 0;
-    int src_p[kFusedSources];
+    // planes on which E has a fused source: [src_lo, src_hi] (empty for nearly every tile)
+    int src_lo = a.Nx, src_hi = -1;
 #pragma unroll
-    for (int s = 0; s < kFusedSources; ++s) {
-        src_p[s] = 0;
-        if (dom && s < a.ns && a.sy[s] == y && a.sz[s] >= z4 && a.sz[s] < z4 + 4) {
-            src_mask |= 1u << s;
-            src_p[s] = a.sz[s] - z4;
+    for (int s = 0; s < kFusedSources; ++s)
+        if (s < a.ns && a.sy[s] >= ye0 && a.sy[s] < ye0 + G::EY && a.sz[s] >= ze0 && a.sz[s] < ze0 + EZ) {
+            src_lo = min(src_lo, a.sx[s]);
+            src_hi = max(src_hi, a.sx[s]);
         }
-    }
 
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     auto load_u = [&](int x) -> float4 {
@@ -162,9 +175,18 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
 #pragma unroll
     for (int j = 1; j <= R; ++j) cz2[j] = f2(a.coef[j], a.coef[j]);
     const int pt_off = ty * EZ + 4 * lz;  // this thread's 4 points in an E plane
-    unsigned amax_bits = 0;
-    bool failed = false;
+    float4 u1q[2 * R + 1];  // OWN_X: the thread's u^{n+1} at planes x - 2R .. x
+#pragma unroll
+    for (int k = 0; k <= 2 * R; ++k) u1q[k] = zero4;
+    float2 nonfinite = f2(0.f, 0.f);
+    // false once this thread's wait has given up: it then runs on without waiting or issuing,
+    // and the results are void (as in tma_segment)
+    bool alive = true;
     int issued = min(S - 1, n_planes), it_failed = 0;
+    // ring planes of u^{n+1}: the slots of planes x - NU1 + 1 .. x, rotated once per plane
+    float *u1p[G::NU1];
+#pragma unroll
+    for (int k = 0; k < G::NU1; ++k) u1p[k] = u1ring + k * (EZ * G::EY);
     int stage = 0;
     uint32_t phase = 0;
 
@@ -174,17 +196,18 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
             const int x = xo + i;
             if (x >= xend) break;
             const int it = x - xs;
-            const bool ok = mbar_wait_bounded(smem_addr(&bars[stage]), phase);
-            if (__syncthreads_or(!ok)) {
-                failed = true;
-                it_failed = it;
-                break;
-            }
-            if (tid == 0 && x + S - 1 < xend) {
+            if (!mbar_try_wait(smem_addr(&bars[stage]), phase))
+                if (alive && !mbar_wait_slow(smem_addr(&bars[stage]), phase)) {
+                    alive = false;
+                    it_failed = it;
+                }
+            __syncthreads();
+            if (tid == 0 && alive && x + S - 1 < xend) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 issue(x + S - 1, stage == 0 ? S - 1 : stage - 1);
                 ++issued;
             }
+            if (tid == 32) prefetch(x + 1 + kPrefetchAhead);
             const unsigned char *st = ring + stage * G::STAGE_BYTES;
             q[2 * R + i] = *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(st + G::OFF_FRONT) + pt_off);
             // ---- step 1: u^{n+1}(x) at this thread's points of E
@@ -209,19 +232,10 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
                 }
                 u1 = tb2_update<R, G::HZ, SW>(rowp, win, [&](int j, bool minus) { return minus ? q[R + i - j] : q[R + i + j]; },
                                              q[R + i], cum, cf1, cf2, cz2);
-                if (src_mask) {
-#pragma unroll
-                    for (int s = 0; s < kFusedSources; ++s) {
-                        if (((src_mask >> s) & 1u) && a.sx[s] == x) {
-                            const float qv = tb2_source(a, s, a.step);
-                            const int p = src_p[s];
-                            if (p == 0) u1.x = fmaf(cf1.x, qv, u1.x);
-                            if (p == 1) u1.y = fmaf(cf1.y, qv, u1.y);
-                            if (p == 2) u1.z = fmaf(cf1.z, qv, u1.z);
-                            if (p == 3) u1.w = fmaf(cf1.w, qv, u1.w);
-                        }
-                    }
-                }
+                if (x >= src_lo && x <= src_hi)
+                    u1 = tma_add_sources<kFactored>(a, u1, x, y, z4, a.step,
+                                                    reinterpret_cast<const float *>(st + G::OFF_F1) + pt_off, nullptr,
+                                                    1.0f);
                 if (z4 + 3 >= a.Nz) {  // beyond the row's end: zero (the Dirichlet halo and the pitch padding)
                     if (z4 + 1 >= a.Nz) u1.y = 0.f;
                     if (z4 + 2 >= a.Nz) u1.z = 0.f;
@@ -229,15 +243,16 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
                 }
                 if (inT && x >= xb && x < xe) *reinterpret_cast<float4 *>(o1 + x * P) = u1;
             }
-            const int slot1 = it % G::NU1;
-            *reinterpret_cast<float4 *>(u1ring + slot1 * (EZ * G::EY) + pt_off) = u1;
+            *reinterpret_cast<float4 *>(u1p[G::NU1 - 1] + pt_off) = u1;
+            if constexpr (G::OWN_X) u1q[2 * R] = u1;
             __syncthreads();  // the ring's plane x is complete
             // ---- step 2: u^{n+2}(x - R) at this thread's points of T
             const int x2 = x - R;
             if (inT && dom && x2 >= xb && x2 < xe) {
-                const int c0 = (it - R) % G::NU1;  // slot of plane x - R
-                const float *plane_c = u1ring + c0 * (EZ * G::EY);
-                const float4 uc = *reinterpret_cast<const float4 *>(plane_c + pt_off);
+                const float *plane_c = u1p[G::NU1 - 1 - R];  // plane x - R
+                float4 uc;
+                if constexpr (G::OWN_X) uc = u1q[R];
+                else uc = *reinterpret_cast<const float4 *>(plane_c + pt_off);
                 const float *rowp = plane_c + ty * EZ + 4 * lz - G::HZ;  // z window from 4 points before
                 float win[NWIN];
 #pragma unroll
@@ -249,50 +264,53 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
                     win[4 * m + 3] = v.w;
                 }
                 auto xtap = [&](int j, bool minus) {
-                    const int sl = (it - R + (minus ? -j : j) + G::NU1) % G::NU1;
-                    return *reinterpret_cast<const float4 *>(u1ring + sl * (EZ * G::EY) + pt_off);
+                    if constexpr (G::OWN_X) return u1q[minus ? R - j : R + j];
+                    else return *reinterpret_cast<const float4 *>(u1p[minus ? R - j : R + j] + pt_off);
                 };
                 const float4 w2 = wq[(i + 1) % U], g2 = gq[(i + 1) % U];  // plane x - R
                 float4 u2 = tb2_update<R, G::HZ, EZ>(rowp, win, xtap, uc, q[i], w2, g2, cz2);
-                if (src_mask) {
-#pragma unroll
-                    for (int s = 0; s < kFusedSources; ++s) {
-                        if (((src_mask >> s) & 1u) && a.sx[s] == x2) {
-                            const float qv = tb2_source(a, s, a.step + 1);
-                            const int p = src_p[s];
-                            if (p == 0) u2.x = fmaf(w2.x, qv, u2.x);
-                            if (p == 1) u2.y = fmaf(w2.y, qv, u2.y);
-                            if (p == 2) u2.z = fmaf(w2.z, qv, u2.z);
-                            if (p == 3) u2.w = fmaf(w2.w, qv, u2.w);
-                        }
-                    }
+                if (x2 >= src_lo && x2 <= src_hi) {
+                    const float w4[4] = {w2.x, w2.y, w2.z, w2.w};
+                    u2 = tma_add_sources<kFactored>(a, u2, x2, y, z4, a.step + 1, w4, nullptr, 1.0f);
                 }
                 if (z4 + 3 >= a.Nz) {
                     if (z4 + 1 >= a.Nz) u2.y = 0.f;
                     if (z4 + 2 >= a.Nz) u2.z = 0.f;
                     if (z4 + 3 >= a.Nz) u2.w = 0.f;
                 }
-                amax_bits = max(amax_bits, max(max(__float_as_uint(fabsf(u2.x)), __float_as_uint(fabsf(u2.y))),
-                                               max(__float_as_uint(fabsf(u2.z)), __float_as_uint(fabsf(u2.w)))));
+                // x * 0 is 0 for finite x and NaN otherwise
+                nonfinite = fma2(lo2(u2), f2(0.f, 0.f), nonfinite);
+                nonfinite = fma2(hi2(u2), f2(0.f, 0.f), nonfinite);
                 *reinterpret_cast<float4 *>(o2 + x2 * P) = u2;
+            }
+            {
+                float *oldest = u1p[0];  // the next plane takes the oldest one's slot
+#pragma unroll
+                for (int k = 0; k < G::NU1 - 1; ++k) u1p[k] = u1p[k + 1];
+                u1p[G::NU1 - 1] = oldest;
+            }
+            if constexpr (G::OWN_X) {
+#pragma unroll
+                for (int k = 0; k < 2 * R; ++k) u1q[k] = u1q[k + 1];
             }
             if (++stage == S) {
                 stage = 0;
                 phase ^= 1u;
             }
         }
-        if (failed) break;
 #pragma unroll
         for (int k = 0; k < 2 * R; ++k) q[k] = q[k + U];
     }
-    if (failed) {
+    if (__syncthreads_or(!alive)) {
         if (tid == 0) {
             if (a.status) atomicOr(a.status, kStatusTimeout);
+            if (alive) it_failed = issued;  // this thread has waited for every copy it issued
             for (int it = it_failed; it < issued; ++it) mbar_wait_bounded(smem_addr(&bars[it % S]), uint32_t(it / S) & 1u);
         }
         return;
     }
-    if (check) reduce_amax(a, amax_bits, false);
+    // as bits: NaN sorts above every finite magnitude (the status test)
+    if (check) reduce_amax(a, nonfinite.x == 0.f && nonfinite.y == 0.f ? 0u : 0x7fc00000u, false);
 }
 
 template <int R>
