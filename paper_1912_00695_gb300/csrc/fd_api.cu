@@ -273,6 +273,7 @@ StepArgs make_args(const fd_handle *hd, long long step, int cur) {
     a.pz = hd->pz;
     a.plane = hd->plane;
     a.x_block = hd->x_block > 0 ? hd->x_block : hd->Nx;
+    a.overlap_launch = hd->slab ? 0 : 1;  // (a slab's steps wait on events of other streams)
     a.x_lo = hd->x_lo;
     a.x_hi = hd->x_hi;
     a.bx0 = hd->box[0];

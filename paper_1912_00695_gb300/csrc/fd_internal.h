@@ -98,6 +98,9 @@ struct StepArgs {
     float *hist;
     float *grad;
     int hist_slot;  // adjoint pass: the history level D^{k-1} sits at
+    // TMA step kernel: launched so that it may start while the previous kernel of its stream
+    // ends (it waits for that kernel before its first access to device memory)
+    int overlap_launch;
 };
 
 // Host numerics (fd_numerics.cpp)

@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
+    wait_previous_launch();
     // the extended tile lies where the damping field vanishes (in y and z)
     const bool tile_yz_box = ye0 >= a.by0 && ye0 + G::EY <= a.by1 && ze0 >= a.bz0 && ze0 + EZ <= a.bz1;
     auto g_free = [&](int x) { return tile_yz_box && x >= a.bx0 && x < a.bx1; };
@@ -325,8 +326,7 @@ cudaError_t tma2_launch(const TmaMaps &maps, const StepArgs &a, float *out1, flo
         attr_set = true;
     }
     const dim3 grid((a.Nz + G::TZ - 1) / G::TZ, (a.Ny + G::TY - 1) / G::TY, (a.Nx + a.x_block - 1) / a.x_block);
-    kernel<<<grid, G::THREADS, G::SMEM_BYTES, s>>>(maps, a, out1, out2, check ? 1 : 0);
-    return cudaGetLastError();
+    return launch_step(kernel, grid, G::THREADS, G::SMEM_BYTES, true, s, maps, a, out1, out2, check ? 1 : 0);
 }
 
 }  // namespace fdgb
