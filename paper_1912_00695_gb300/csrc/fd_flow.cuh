@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(32 * W, (tma_warps_per_sm(R) / W > 0 ? tma_war
         }
         const int xb = it.w * sa.x_block;
         TmaAcc acc;
-        if (!tma_segment<R, FORM, LZ, W, float, kModeStep, true>(s_maps, sa, sc, it.y, it.z, xb,
+        if (!tma_segment<R, FORM, LZ, W, float, kModeStep, true, 1, false>(s_maps, sa, sc, it.y, it.z, xb,
                                                                  min(xb + sa.x_block, sa.Nx), ring, g, acc, nullptr,
                                                                  s_step)) {
             ok_all = false;  // a ring wait gave up (status set); the ring's phases are no longer known

@@ -213,7 +213,8 @@ __global__ void __launch_bounds__(128, NoallocShape<R>::CTAS) noalloc_step_kerne
             float win[NWIN];
 #pragma unroll
             for (int m = 0; m < NWIN / 4; ++m) {
-                const float4 v = *reinterpret_cast<const float4 *>(rowp + 4 * m);
+                // (the window's middle is the thread's own points)
+                const float4 v = 4 * m == RZ ? q[R + i] : *reinterpret_cast<const float4 *>(rowp + 4 * m);
                 win[4 * m] = v.x, win[4 * m + 1] = v.y, win[4 * m + 2] = v.z, win[4 * m + 3] = v.w;
             }
             const float2 hdt = pair(half_dt), ucA = lo2(q[R + i]), ucB = hi2(q[R + i]);

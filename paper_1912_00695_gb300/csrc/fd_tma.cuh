@@ -306,7 +306,8 @@ static __device__ __noinline__ float4 tma_add_sources(const StepArgs &a, float4 
 // and meets one CTA barrier per 8 points instead of 4; its x queues take
 // twice the registers, so such CTAs run at half the warps per SM. The
 // per-point arithmetic and its order are those of one row per thread.
-template <int R, int FORM, int LZ, int W, typename T, int MODE = kModeStep, bool COHERENT = false, int YB = 1>
+template <int R, int FORM, int LZ, int W, typename T, int MODE = kModeStep, bool COHERENT = false, int YB = 1,
+          bool OWN_CENTRE = YB == 1>
 __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs &a, const ScaleState &sc, int bz,
                                             int by, int xb, int xe, unsigned char *ring, int &g, TmaAcc &acc,
                                             const GradMaps *gm = nullptr, long long step = -1) {
@@ -490,20 +491,26 @@ __device__ __forceinline__ bool tma_segment(const TmaMaps *maps, const StepArgs 
                 const T *t = reinterpret_cast<const T *>(st);
                 const T *rowp = t + (ty + R) * SW + colw;  // the first row's window in the halo tile
                 const bool gf = g_free(x);
+                float4 uc[YB];
+#pragma unroll
+                for (int r = 0; r < YB; ++r) uc[r] = q[r][R + i];
+                // z windows; their middle four values are the row's own points, which the x
+                // queue already holds (OWN_CENTRE): one shared load less of 10 to 24 per row and plane
+                // (276^3, flow: space order 8 / 12 / 16 factored 366.5 / 303.5 / 268.0 -> 367.4 /
+                // 308.6 / 270.3 Gpts/s, 8 expanded 288.2 -> 290.5, 12 / 4 in BF16 239.8 / 423.4 ->
+                // 242.8 / 429.0; not with two rows per thread, where FP16 lost 1.7 %, nor in the
+                // persistent batch kernel: 12 uneven shots at 8 325 -> 299)
                 float win[YB][NWIN];
 #pragma unroll
                 for (int r = 0; r < YB; ++r)
 #pragma unroll
                     for (int m = 0; m < NWIN / 4; ++m) {
-                        const float4 v = V::ld(rowp + r * SW + 4 * m);
+                        const float4 v = OWN_CENTRE && 4 * m == RZ ? uc[r] : V::ld(rowp + r * SW + 4 * m);
                         win[r][4 * m] = v.x;
                         win[r][4 * m + 1] = v.y;
                         win[r][4 * m + 2] = v.z;
                         win[r][4 * m + 3] = v.w;
                     }
-                float4 uc[YB];
-#pragma unroll
-                for (int r = 0; r < YB; ++r) uc[r] = q[r][R + i];
                 // the y taps at distance j of row r: ym(r, j) = row r - j, yp(r, j) = row r + j.
                 // Two rows share the loads: iteration j loads rows -j and j + 1 (relative to
                 // the first row) and keeps rows j and 1 - j from the previous iteration

@@ -225,7 +225,8 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
                 float win[NWIN];
 #pragma unroll
                 for (int m = 0; m < NWIN / 4; ++m) {
-                    const float4 v = *reinterpret_cast<const float4 *>(rowp + 4 * m);
+                    // (the window's middle is the thread's own points)
+                    const float4 v = 4 * m == G::HZ ? q[R + i] : *reinterpret_cast<const float4 *>(rowp + 4 * m);
                     win[4 * m] = v.x;
                     win[4 * m + 1] = v.y;
                     win[4 * m + 2] = v.z;
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(256, 2) fd_tma2_kernel(const __grid_constant__
                 float win[NWIN];
 #pragma unroll
                 for (int m = 0; m < NWIN / 4; ++m) {
-                    const float4 v = *reinterpret_cast<const float4 *>(rowp + 4 * m);
+                    const float4 v = 4 * m == G::HZ ? uc : *reinterpret_cast<const float4 *>(rowp + 4 * m);
                     win[4 * m] = v.x;
                     win[4 * m + 1] = v.y;
                     win[4 * m + 2] = v.z;
