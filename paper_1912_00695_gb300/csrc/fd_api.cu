@@ -1626,13 +1626,14 @@ int fd_forward(fd_handle *hd, int nt) {
     if (!hd->has_model) return fail(FD_ESTATE, "fd_forward before fd_set_model");
     if (nt == 0) return FD_OK;
     // automatic kernel choice, space order 2: two steps per launch where the single-step
-    // kernel is bound by HBM traffic (measured 1.15x at 276^3; at space order 4 the
-    // overlap of the extended tiles costs more than the traffic saved). Same bits.
+    // kernel is bound by HBM traffic (276^3: 455 to 481 Gpts/s against the 389 of the
+    // single-step kernel's expanded form, its nearest; at space order 4 360 against the
+    // flow's 382: the overlap of the extended tiles costs more than the traffic saved). Same bits.
     if (nt >= 2 && hd->opt.kernel == kAuto && hd->kernel == kTma && hd->r == 1 && hd->opt.storage == kF32 &&
         hd->opt.form == kFactored && hd->n_rec == 0 && int(hd->sources.size()) <= kFusedSources)
         return fd_forward_two_step(hd, nt);
     // automatic kernel choice, FP32 otherwise: the flow schedule (one persistent launch,
-    // no per-step tail or launch gap; measured 1.02-1.10x over per-step launches at
+    // no per-step tail or launch gap; measured 1.12-1.21x over per-step launches at
     // 276^3 for every space order and form) where it was timed faster than the per-step
     // launches for this grid. Same bits either way.
     if (hd->opt.kernel == kAuto && flow_eligible(hd)) {
