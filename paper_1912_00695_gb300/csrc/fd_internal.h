@@ -26,13 +26,14 @@ constexpr int kModeStep = 0, kModeForwardD = 1, kModeAdjointGrad = 2;
 // at R = 8).
 constexpr int kTmaWarpsPerSM = 16;
 // Above radius 8 the register queue needs more than 128 registers per thread. Radii 9 and 10
-// factored are compiled for 8 warps per SM and fit 12 by themselves; radii 11 and 12, and the
-// expanded form, are held to the 168 registers that 12 warps leave (276^3, flow, held / not:
-// space order 24 factored 188.3 / 161.2 Gpts/s, expanded 135.4 / 120.8, in BF16 151.7 / 134.3;
-// but 18 and 20 factored 221.1 / 235.8 and 209.5 / 221.2).
+// factored and 9 expanded are compiled for 8 warps per SM and fit 12 by themselves; radii 11
+// and 12, and 10 expanded, are held to the 168 registers that 12 warps leave (276^3, flow,
+// held / not: space order 24 factored 188.3 / 161.2 Gpts/s, expanded 135.4 / 120.8, in BF16
+// 151.7 / 134.3, 20 expanded at 220^3 149.4 / 129.2; but 18 and 20 factored 221.1 / 235.8 and
+// 209.5 / 221.2, 18 expanded 166.2 / 171.7).
 // Two y rows per thread double the x queues: 8 warps per SM.
 constexpr int tma_warps_per_sm(int r, int rows = 1, int form = 0) {
-    return rows > 1 ? 8 : r <= 8 ? kTmaWarpsPerSM : r > 10 || form != 0 ? 12 : 8;
+    return rows > 1 ? 8 : r <= 8 ? kTmaWarpsPerSM : r > 10 || (form != 0 && r > 9) ? 12 : 8;
 }
 constexpr int kTileZ = 32;          // streaming tile width along z (one warp)
 constexpr int kMaxDim = 65535;  // keeps every launch grid dimension within limits
