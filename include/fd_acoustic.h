@@ -269,8 +269,8 @@ int fd_forward_two_step(fd_handle *hd, int nt);
  * shape (candidates 8-64 planes, 8 steps each; all of them part of the
  * requested steps, same bits) and cached for the process; a shorter first
  * call takes the multiple of 4 planes, up to 40, that gives about 1.7 items a
- * step per resident CTA (and fd_forward runs the per-step launches for 16 steps
- * and more where that is below 6 planes) for that call only. The same first call compares the
+ * step per resident CTA (and fd_forward runs an FP32 shot's per-step launches for
+ * 16 steps and more where that is below 6 planes) for that call only. The same first call compares the
  * two schedules by the cost of one more step: the best length and the
  * per-step launches each run 8 and 24 steps, and (t24 - t8) / 16 is compared,
  * which cancels a launch's start-up and last tail.

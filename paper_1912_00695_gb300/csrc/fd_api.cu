@@ -1995,8 +1995,10 @@ static int flow_prepare(fd_handle *hd, int *nt) {
         // 56^3 3.1 / 4.4 per step against 6.5 / 12.5 flow at best (40-plane items 20 / 31),
         // 84^3 5.3 / 7.5 against 5.0 / 13.3 (26 / 44), 150^3 12.2 / 21.2 against 11.9 / 17.3.
         // Calls of fewer than 16 steps stay one flow launch: recording and instantiating
-        // their per-step graph would cost more than their steps.
-        hd->flow_wins = even >= 6.0 || *nt < 16;
+        // their per-step graph would cost more than their steps. So do BF16 shots: the flow
+        // stores levels unscaled, and values that are subnormal in one schedule and not in the
+        // other can break a rounding tie, after which the two part by BF16's own noise.
+        hd->flow_wins = even >= 6.0 || *nt < 16 || hd->opt.storage != kF32;
         const int xb = 4 * std::max(1, std::min(10, int(even / 4.0 + 0.5)));
         return use(std::min(hd->Nx, std::max(xb, hd->r)));
     }
