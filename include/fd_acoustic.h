@@ -253,7 +253,13 @@ int fd_forward_two_step(fd_handle *hd, int nt);
  * are taken in step order by resident CTAs, and an item starts as soon as the
  * 27 items of the previous step around it are done, so the SMs do not idle in
  * the tail of each step and between launches. Same per-point arithmetic as
- * fd_forward with the TMA kernel: the same results bit for bit. FP32 storage
+ * fd_forward with the TMA kernel: the same results bit for bit in FP32 storage.
+ * In BF16 this schedule stores levels unscaled where per-step launches scale
+ * them by powers of two: the values agree except where one is subnormal and the
+ * other is not, far ahead of the wave front (below 1e-20 of the field's maximum),
+ * which over hundreds of steps can break a rounding tie; from there the two fields
+ * part by BF16's own noise (measured rel-L2 up to 2.5e-2 after 285 steps, each
+ * 2.6e-2 from the 64-bit result). FP32 storage
  * (BF16 with at most 4 sources and no receivers), the TMA kernel (either
  * form), zero boundary, x_block >= k/2 (FD_ENOTSUP otherwise). With FP32,
  * receivers and sources beyond the 4 fused ones ride on the items: an item
@@ -277,7 +283,11 @@ int fd_forward_two_step(fd_handle *hd, int nt);
  * fd_forward takes this path when the kernel is left to the library
  * (FD_KERNEL_AUTO), the conditions hold, the two-step path (space order 2,
  * factored) does not apply and that comparison did not find the per-step
- * launches cheaper per step for the grid.
+ * launches cheaper per step for the grid. For BF16 no timing decides: fd_forward
+ * takes this path, except on small grids (N_x ceil(N_y/16) ceil(N_z/32) below 34
+ * times the multiprocessors, 47.6 at space orders 22 and 24: up to about 128^3 and
+ * 144^3 points) from the first call of at least 144 steps since a reset or a loaded
+ * state on; there it runs per-step launches. The x-chunk never changes a bit.
  * Asynchronous like fd_forward; fd_last_forward_ms times the launch. */
 int fd_forward_flow(fd_handle *hd, int nt);
 
@@ -294,11 +304,12 @@ int fd_read_traces(fd_handle *hd, float *out, int *recorded);
  * t0, t1, t2 (Sec. 2.1); the paper's measured runs repeat it 30,000 times
  * (Sec. 4). The global step counter persists across calls, so
  * fd_forward(a) followed by fd_forward(b) equals fd_forward(a + b) bit for
- * bit. Steps are replayed from a cached CUDA graph. With the kernel left to
- * the library, FP32 shots run the flow schedule (fd_forward_flow) or, at
- * space order 2 factored without receivers, two steps per launch
- * (fd_forward_two_step); every schedule gives the same bits. FD_ESTATE
- * without a model; FD_EINVAL for nt < 0. */
+ * bit (BF16 with the kernel left to the library: where both run one schedule,
+ * see fd_forward_flow). Steps are replayed from a cached CUDA graph. With the
+ * kernel left to the library, FP32 and BF16 shots run the flow schedule
+ * (fd_forward_flow) or, FP32 at space order 2 factored without receivers, two
+ * steps per launch (fd_forward_two_step); every schedule gives the same bits in
+ * FP32. FD_ESTATE without a model; FD_EINVAL for nt < 0. */
 int fd_forward(fd_handle *hd, int nt);
 
 /* Copy a wavefield level to a HOST array of N_x*N_y*N_z floats (dense C-order;

@@ -66,8 +66,9 @@ std::map<std::tuple<int, int, int, int, int, int, int, int>, std::tuple<int, int
 std::map<std::tuple<int, int, int, int>, int> g_tb_cache;
 // FWI gradient passes: (Nx, Ny, Nz, radius) -> x_block of the forward and of the adjoint pass
 std::map<std::tuple<int, int, int, int>, std::pair<int, int>> g_grad_cache;
-// flow schedule: (Nx, Ny, Nz, radius, form, tile_z, tile_y) -> (x_block, faster than per-step launches)
-std::map<std::tuple<int, int, int, int, int, int, int, int>, std::pair<int, bool>> g_flow_cache;
+// flow schedule: (Nx, Ny, Nz, radius, storage, form, tile_z, tile_y, rows, extras) -> (x_block, faster
+// than per-step launches; BF16 takes the x_block alone)
+std::map<std::tuple<int, int, int, int, int, int, int, int, int, int>, std::pair<int, bool>> g_flow_cache;
 
 // Device memory is stream-ordered (cudaMallocAsync / cudaFreeAsync) from the
 // device's default pool, whose release threshold is raised once per device so
@@ -215,7 +216,8 @@ struct fd_handle {
     int flow_ctas = 0, flow_ctas_ex = 0;  // resident CTAs: plain flow kernel / receivers + extra sources variant
     int flow_xb = 0;         // the flow schedule's x_block, timed, cached or forced (0: not yet)
     int flow_run_xb = 0;     // the x_block the flow graphs are recorded with
-    bool flow_wins = true;   // the flow beat per-step launches when the two were timed
+    bool flow_wins = true;   // the flow beat per-step launches when the two were timed (BF16: by rule)
+    bool long_run = false;   // BF16: an fd_forward of at least 144 steps since the last reset
     int flow_extras = -1;    // receivers (1) / extra sources (2) present when flow_xb was chosen
     struct TbMaps {
         const void *u, *up;
@@ -1617,7 +1619,7 @@ static int ensure_step_tuned(fd_handle *hd);
 static int run_steps(fd_handle *hd, int nt);
 static int run_flow(fd_handle *hd, int nt);
 static bool flow_eligible(const fd_handle *hd);
-static int flow_prepare(fd_handle *hd, int *nt);
+static int flow_prepare(fd_handle *hd, int *nt, bool flow_only);
 
 int fd_forward(fd_handle *hd, int nt) {
     if (!hd) return fail(FD_EINVAL, "handle is NULL");
@@ -1632,12 +1634,12 @@ int fd_forward(fd_handle *hd, int nt) {
     if (nt >= 2 && hd->opt.kernel == kAuto && hd->kernel == kTma && hd->r == 1 && hd->opt.storage == kF32 &&
         hd->opt.form == kFactored && hd->n_rec == 0 && int(hd->sources.size()) <= kFusedSources)
         return fd_forward_two_step(hd, nt);
-    // automatic kernel choice, FP32 otherwise: the flow schedule (one persistent launch,
+    // automatic kernel choice otherwise: the flow schedule (one persistent launch,
     // no per-step tail or launch gap; measured 1.12-1.21x over per-step launches at
     // 276^3 for every space order and form) where it was timed faster than the per-step
-    // launches for this grid. Same bits either way.
+    // launches for this grid (FP32: same bits either way) or the rule for BF16 says so.
     if (hd->opt.kernel == kAuto && flow_eligible(hd)) {
-        int rc = flow_prepare(hd, &nt);
+        int rc = flow_prepare(hd, &nt, false);
         if (rc != FD_OK || nt == 0) return rc;
         return hd->flow_wins ? run_flow(hd, nt) : run_steps(hd, nt);
     }
@@ -1936,11 +1938,23 @@ static bool flow_eligible(const fd_handle *hd) {
            hd->opt.boundary == FD_BOUNDARY_ZERO && (hd->opt.x_block == 0 || hd->opt.x_block >= hd->r);
 }
 
-// Chooses the flow schedule's x_block and whether it beats per-step launches,
-// timing the candidates on the first steps of this call (*nt is reduced by the
-// steps they ran; every candidate computes the same bits). Cached per grid and
-// launch shape for the process.
-static int flow_prepare(fd_handle *hd, int *nt) {
+// Chooses the flow schedule's x_block and whether fd_forward runs it or per-step
+// launches (flow_only: the caller runs the flow), timing the candidates on the first
+// steps of this call (*nt is reduced by the steps they ran). Cached per grid, storage
+// and launch shape for the process. FP32: every candidate computes the same bits. BF16:
+// the same bits at any x_block, but the flow stores levels unscaled and per-step launches
+// scale them, and a value that is subnormal in one and not in the other can break a
+// rounding tie, after which the two fields part by BF16's own noise (rel-L2 2.5e-2 at
+// 106x103x99, space order 12, 285 steps, each 2.6e-2 from the 64-bit result). So a BF16
+// shot's schedule never follows a timing or another shot: it is the flow, except that from
+// the first fd_forward of at least 144 steps since a reset on (what timing takes in FP32),
+// grids of fewer than 5 planes per item (7 at space orders 22 and 24) run per-step launches,
+// counted in 32x16 tiles at four CTAs per multiprocessor, so that the tuned tile has no say.
+// One GB300, 200 steps, us a step per-step / flow at space orders 4, 8, 16, 24: 56^3 4.7 / 8.2,
+// 4.3 / 8.3, 5.1 / 13.1, -; 120^3 (3.7 planes) 8.5 / 11.4, 9.7 / 10.6, 13.3 / 16.6, 18.9 / 22.7;
+// 130^3 (5.7) 11.0 / 9.8, 13.8 / 12.7, 19.1 / 19.1, 24.6 / 27.0; 150^3 (7.3) 12.8 / 12.7,
+// 16.4 / 15.3, 23.2 / 20.5, 30.1 / 29.4.
+static int flow_prepare(fd_handle *hd, int *nt, bool flow_only) {
     int rc = ensure_step_tuned(hd);
     if (rc != FD_OK) return rc;
     // the x_block the graphs use follows the chosen one
@@ -1951,9 +1965,17 @@ static int flow_prepare(fd_handle *hd, int *nt) {
         }
         return FD_OK;
     };
+    const bool by_rule = hd->opt.storage != kF32;
     // receivers and extra sources change the balance of the two schedules: their
     // presence is part of the choice (made again when it changes)
     const int extras = (hd->n_rec > 0 ? 1 : 0) | (int(hd->sources.size()) > kFusedSources ? 2 : 0);
+    if (by_rule && !flow_only) {
+        hd->long_run |= *nt >= 144;
+        const double items = double((hd->Nz + 31) / 32) * double((hd->Ny + 15) / 16);
+        hd->flow_wins = hd->opt.x_block > 0 || !hd->long_run ||
+                        double(hd->Nx) * items / (1.7 * 4.0 * device_sms()) >= (hd->r > 10 ? 7.0 : 5.0);
+        if (!hd->flow_wins) return FD_OK;
+    }
     if (hd->flow_xb != 0 && hd->flow_extras == extras) return use(hd->flow_xb);
     hd->flow_extras = extras;
     if (hd->opt.x_block > 0) {  // forced by the options
@@ -1962,23 +1984,24 @@ static int flow_prepare(fd_handle *hd, int *nt) {
         return use(hd->flow_xb);
     }
     hd->flow_xb = 0;
-    const auto key = std::make_tuple(hd->Nx, hd->Ny, hd->Nz, hd->r, hd->opt.form, hd->tile_z, hd->tile_y, extras);
+    const auto key = std::make_tuple(hd->Nx, hd->Ny, hd->Nz, hd->r, hd->opt.storage, hd->opt.form, hd->tile_z,
+                                     hd->tile_y, hd->rows, extras);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_flow_cache.find(key);
         if (it != g_flow_cache.end()) {
             hd->flow_xb = it->second.first;
-            hd->flow_wins = it->second.second;
+            if (!by_rule) hd->flow_wins = it->second.second;
             return use(hd->flow_xb);
         }
     }
-    // shorter x-chunks balance better and keep more items in flight on small grids,
-    // longer ones claim fewer items and re-read fewer queue planes
-    constexpr int kTuneSteps = 8, kLongSteps = 24;
     // the x-chunk that gives about 1.7 items a step for each resident CTA: the items of a
     // step then overlap the last step's tail, and no CTA carries a long chain of planes alone
     const long long tiles = (long long)((hd->Nz + hd->tile_z - 1) / hd->tile_z) * ((hd->Ny + hd->tile_y - 1) / hd->tile_y);
     const double even = double(hd->Nx) * double(tiles) / (1.7 * std::max(1, flow_slots(hd, hd->opt.storage == kF32 && extras != 0)));
+    // shorter x-chunks balance better and keep more items in flight on small grids,
+    // longer ones claim fewer items and re-read fewer queue planes
+    constexpr int kTuneSteps = 8, kLongSteps = 24;
     std::vector<int> cand;
     for (int c : {8, 12, 16, 24, 32, 40, 48, 56, even < 8.0 ? 4 : 64})
         if (c >= hd->r && c <= hd->Nx) cand.push_back(c);
@@ -1995,10 +2018,8 @@ static int flow_prepare(fd_handle *hd, int *nt) {
         // 56^3 3.1 / 4.4 per step against 6.5 / 12.5 flow at best (40-plane items 20 / 31),
         // 84^3 5.3 / 7.5 against 5.0 / 13.3 (26 / 44), 150^3 12.2 / 21.2 against 11.9 / 17.3.
         // Calls of fewer than 16 steps stay one flow launch: recording and instantiating
-        // their per-step graph would cost more than their steps. So do BF16 shots: the flow
-        // stores levels unscaled, and values that are subnormal in one schedule and not in the
-        // other can break a rounding tie, after which the two part by BF16's own noise.
-        hd->flow_wins = even >= 6.0 || *nt < 16 || hd->opt.storage != kF32;
+        // their per-step graph would cost more than their steps.
+        if (!by_rule) hd->flow_wins = even >= 6.0 || *nt < 16;
         const int xb = 4 * std::max(1, std::min(10, int(even / 4.0 + 0.5)));
         return use(std::min(hd->Nx, std::max(xb, hd->r)));
     }
@@ -2013,21 +2034,27 @@ static int flow_prepare(fd_handle *hd, int *nt) {
             best_xb = c;
         }
     }
-    // schedule choice by differential timing: the cost of one more step, (t_long -
-    // t_short) / (kLongSteps - kTuneSteps), for both schedules. A flow launch carries a
-    // start-up and a last tail that a long run spreads out; the difference cancels them
-    // (and the per-step launches' first-launch overhead) instead of a hand-set margin.
-    // Both lengths are timed afresh: the candidates' minimum is biased low.
-    if (rc == FD_OK) rc = flow_direct(hd, kTuneSteps, best_xb, &flow_short);
-    if (rc == FD_OK) rc = flow_direct(hd, kLongSteps, best_xb, &flow_long);
-    if (rc == FD_OK) rc = steps_direct(hd, kTuneSteps, &step_short);
-    if (rc == FD_OK) rc = steps_direct(hd, kLongSteps, &step_long);
+    int taken = kTuneSteps * (int(cand.size()) + 1);
+    if (!by_rule) {
+        // schedule choice by differential timing: the cost of one more step, (t_long -
+        // t_short) / (kLongSteps - kTuneSteps), for both schedules. A flow launch carries a
+        // start-up and a last tail that a long run spreads out; the difference cancels them
+        // (and the per-step launches' first-launch overhead) instead of a hand-set margin.
+        // Both lengths are timed afresh: the candidates' minimum is biased low.
+        if (rc == FD_OK) rc = flow_direct(hd, kTuneSteps, best_xb, &flow_short);
+        if (rc == FD_OK) rc = flow_direct(hd, kLongSteps, best_xb, &flow_long);
+        if (rc == FD_OK) rc = steps_direct(hd, kTuneSteps, &step_short);
+        if (rc == FD_OK) rc = steps_direct(hd, kLongSteps, &step_long);
+        taken = needed;
+    }
     if (rc != FD_OK) return rc;
-    *nt -= needed;
+    *nt -= taken;
     hd->flow_xb = best_xb;
-    const float flow_per_step = (flow_long - flow_short) / float(kLongSteps - kTuneSteps);
-    const float steps_per_step = (step_long - step_short) / float(kLongSteps - kTuneSteps);
-    hd->flow_wins = flow_per_step <= steps_per_step;
+    if (!by_rule) {
+        const float flow_per_step = (flow_long - flow_short) / float(kLongSteps - kTuneSteps);
+        const float steps_per_step = (step_long - step_short) / float(kLongSteps - kTuneSteps);
+        hd->flow_wins = flow_per_step <= steps_per_step;
+    }
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         g_flow_cache[key] = std::make_pair(hd->flow_xb, hd->flow_wins);
@@ -2049,7 +2076,7 @@ int fd_forward_flow(fd_handle *hd, int nt) {
     if (hd->opt.x_block > 0 && hd->opt.x_block < hd->r)
         return fail(FD_ENOTSUP, "the flow schedule needs x_block >= k/2");
     if (nt == 0) return FD_OK;
-    int rc = flow_prepare(hd, &nt);
+    int rc = flow_prepare(hd, &nt, true);
     if (rc != FD_OK || nt == 0) return rc;
     return run_flow(hd, nt);
 }
@@ -2150,6 +2177,7 @@ int fd_load_state(fd_handle *hd, const float *u, const float *u_prev, long long 
     }
     hd->rec_step0 = step;
     hd->step = step;
+    hd->long_run = false;
     hd->cur = 0;
     return FD_OK;
 }
@@ -2167,6 +2195,7 @@ int fd_reset(fd_handle *hd) {
     hd->rec_step0 = 0;
     hd->step = 0;
     hd->cur = 0;
+    hd->long_run = false;
     return FD_OK;
 }
 
