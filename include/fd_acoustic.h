@@ -217,7 +217,10 @@ int fd_set_receivers(fd_handle *hd, int n, const double *xyz, int nt_max);
  * arguments, FD_ESTATE without a model, FD_ENOTSUP for other storage/form/
  * kernel choices. Synchronises; fd_last_forward_ms then returns the device
  * time of the two passes (which run back to back: the residual is formed on
- * the device). When the history does not fit in 80 % of the free device
+ * the device). Each pass's x-chunk is the options' x_block if set, else the one
+ * timed fastest on the steps of the grid's first pass that is long enough (same
+ * bits; the waits between its first steps count in that call's time), the step
+ * kernel's until then. When the history does not fit in 80 % of the free device
  * memory, the call checkpoints instead (as fd_fwi_gradient_checkpointed with
  * segment = ceil(sqrt(nt))). */
 int fd_fwi_gradient(fd_handle *hd, int nrec, const double *rec_xyz, const float *d_obs, int nt, float *grad_out,

@@ -16,6 +16,7 @@
 #include "../../include/fd_acoustic.h"
 #include "fd_internal.h"
 #include "fd_flow.h"
+#include "fd_grad_chunks.h"
 #include "fd_launch_count.h"
 #include "fd_periodic.h"
 
@@ -1112,10 +1113,17 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
     const int nseg = (nt + segment - 1) / segment;
     const bool ckpt = nseg > 1;
     const int tz = 32, ty = 16;  // the gradient passes' tile
-    // x-chunk of each pass (0: not chosen yet)
+    // x-chunk of each pass (0: not chosen yet): the options' if they name one, else timed; a pass
+    // too short to time takes the step kernel's (one GB300, 14 steps, us a step of both passes at
+    // two CTAs per multiprocessor -> the step's chunk: 84^3 at space order 4 26.2 -> 18.1, 200^3
+    // at 16 116 -> 102, 276^3 at 8 / 16 / 24 219 / 279 / 344 -> 215 / 226 / 279)
     const auto xb_key = std::make_tuple(hd->Nx, hd->Ny, hd->Nz, hd->r);
+    const char *no_tune = std::getenv("FDGB_NO_TUNE");
+    const std::vector<int> chunks =
+        grad_chunks(hd->Nx, (long long)((hd->Nz + tz - 1) / tz) * ((hd->Ny + ty - 1) / ty), device_sms(),
+                    hd->opt.x_block, hd->x_block, !(no_tune && no_tune[0] == '1'));
     std::pair<int, int> xbs(0, 0);
-    {
+    if (hd->opt.x_block == 0) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_grad_cache.find(xb_key);
         if (it != g_grad_cache.end()) xbs = it->second;
@@ -1226,41 +1234,28 @@ static int fwi_gradient_impl(fd_handle *hd, int nrec, const double *rec_xyz, con
     // plain step's chunk -> timed ones: 150^3 48.5 -> 41.8, 200^3 101.0 -> 90.6, 276^3 194.5 -> 192.2.
     auto run_pass = [&](int count, int &chosen, auto &&launch) {
         cudaError_t err = cudaSuccess;
-        const int fallback = heuristic_x_block(hd, tz, ty);
         int i = 0;
-        if (chosen == 0) {
-            const long long tiles = (long long)((hd->Nz + tz - 1) / tz) * ((hd->Ny + ty - 1) / ty);
-            std::vector<int> cand = {fallback};  // (a warm-up: timed again below)
-            auto add = [&](long long c) {
-                if (c >= 1 && c <= hd->Nx && std::find(cand.begin() + 1, cand.end(), int(c)) == cand.end())
-                    cand.push_back(int(c));
-            };
-            for (int c : {12, 16, 20, 32, 64}) add(c);
-            for (int ctas : {3, 4, 6, 8}) {  // per SM: one and two waves
-                const long long chunks = (long long)ctas * device_sms() / tiles;
-                if (chunks >= 1) add((hd->Nx + chunks - 1) / chunks);
-            }
-            if (cand.size() == 1) cand.push_back(hd->Nx);
+        if (chosen == 0 && chunks.size() > 1) {
             constexpr int kPer = 2;
-            if (count >= kPer * int(cand.size())) {
+            if (count >= kPer * int(chunks.size())) {
                 for (int k = 0; k < 2 && err == cudaSuccess; ++k)
                     if (!tune_ev[k]) err = cudaEventCreate(&tune_ev[k]);
                 float best = 1e30f;
-                for (size_t c = 0; c < cand.size() && err == cudaSuccess; ++c) {
+                for (size_t c = 0; c < chunks.size() && err == cudaSuccess; ++c) {
                     err = cudaEventRecord(tune_ev[0], st);
-                    for (int k = 0; k < kPer && err == cudaSuccess; ++k) err = launch(i++, cand[c]);
+                    for (int k = 0; k < kPer && err == cudaSuccess; ++k) err = launch(i++, chunks[c]);
                     if (err == cudaSuccess) err = cudaEventRecord(tune_ev[1], st);
                     if (err == cudaSuccess) err = cudaEventSynchronize(tune_ev[1]);
                     float ms = 0.0f;
                     if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, tune_ev[0], tune_ev[1]);
                     if (c > 0 && err == cudaSuccess && ms < best) {
                         best = ms;
-                        chosen = cand[c];
+                        chosen = chunks[c];
                     }
                 }
             }
         }
-        const int xb = chosen > 0 ? chosen : fallback;
+        const int xb = chosen > 0 ? chosen : chunks[0];
         for (; i < count && err == cudaSuccess; ++i) err = launch(i, xb);
         return err;
     };
