@@ -6,9 +6,19 @@
 
 namespace fdgb {
 
-// Passes `e` through; on success counts `n` launches on stream `s` (as recorded
-// into this thread's graph if `s` is capturing, else as executed).
-cudaError_t counted(cudaError_t e, cudaStream_t s, int n = 1);
+// Counts `n` launches on stream `s` (as recorded into this thread's graph if `s`
+// is capturing, else as executed).
+void count_launches(cudaStream_t s, int n);
+// Passes `e` through; on success counts `n` launches. A launch that failed is its
+// caller's error alone: the runtime's last error is cleared, so that the next
+// launch, of whichever handle, does not report it again.
+inline cudaError_t counted(cudaError_t e, cudaStream_t s, int n = 1) {
+    if (e == cudaSuccess)
+        count_launches(s, n);
+    else
+        cudaGetLastError();
+    return e;
+}
 // Launches this thread has recorded into graphs so far.
 long long captured_launches();
 // A replay of a graph holding `n` launches.

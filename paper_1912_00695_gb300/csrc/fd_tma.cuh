@@ -760,8 +760,8 @@ __device__ __forceinline__ void tma_finish(TmaAcc &acc, const ScaleState &sc) {
 __device__ __forceinline__ void wait_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Launches a step kernel; `overlap`: its launch may be processed while the stream's previous
-// kernel ends (the kernel calls wait_previous_launch). A launch that fails is this caller's
-// error alone: it is cleared, so that the next launch, of whichever handle, does not report it.
+// kernel ends (the kernel calls wait_previous_launch). A launch that fails leaves the runtime's
+// last error set: the launcher's counted() clears it.
 template <typename K, typename... A>
 cudaError_t launch_step(K kernel, dim3 grid, int threads, int smem, bool overlap, cudaStream_t s, const A &...args) {
     cudaLaunchConfig_t cfg{};
@@ -774,9 +774,7 @@ cudaError_t launch_step(K kernel, dim3 grid, int threads, int smem, bool overlap
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = overlap ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
-    if (e != cudaSuccess) cudaGetLastError();
-    return e;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Receivers of a single-shot step: every thread of the grid samples at most a
