@@ -591,7 +591,7 @@ int fd_slab_exchange(fd_handle *from, fd_handle *to, int level, void *stream);
  * pieces of four (two) floats. The first call on a
  * device looks up that device's copy of the array (cudaGetSymbolAddress) and
  * its multiprocessor count (which sizes the x-chunks: four CTAs per
- * multiprocessor) once; make that first call before any stream capture. Every call on a device
+ * multiprocessor, three above space order 10) once; make that first call before any stream capture. Every call on a device
  * shares the same array and clears the running maximum at its start, so calls
  * that overlap on the GPU (other streams, other threads) race on it.
  *

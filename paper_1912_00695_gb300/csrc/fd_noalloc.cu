@@ -24,7 +24,7 @@ void set_last_error(const char *msg);  // fd_api.cu: the fd_last_error() text
 
 namespace {
 
-constexpr int kNoAllocMaxCtas = 16384;  // 32x8 tiles a y-z plane may hold (a documented limit)
+constexpr int kNoAllocMaxTiles = 16384;  // 8 x 32 tiles a y-z plane may hold (a documented limit)
 constexpr int kNoAllocMaxDevices = 64;
 
 // Scratch: word 0 = running max |u| (float bits) over the call's steps. Held by
@@ -49,6 +49,11 @@ __device__ __forceinline__ void copy_async(uint32_t dst, const float *src, bool 
 
 __device__ __forceinline__ float2 pair(float v) { return make_float2(v, v); }
 
+// CTAs of the step kernel per multiprocessor. Above radius 5 four would leave 128 registers a
+// thread and spills (one GB300, 186^3 damped, 150 steps: space order 12 69.9 us a step at four,
+// 62.3 at three; 16 81.8 and 70.8)
+constexpr int noalloc_ctas_per_sm(int r) { return r <= 5 ? 4 : 3; }
+
 template <int R>
 struct NoallocShape {
     static constexpr int TZ = 32, TY = 16, W = 4;  // tile: 8 x 4 threads of 4 z points per warp
@@ -57,9 +62,6 @@ struct NoallocShape {
     static constexpr int HALO = SW * SH, PT = TZ * TY;  // floats
     static constexpr int STAGE = HALO + 4 * PT;         // halo tile, front, u^{n-1}, m, eta
     static constexpr int S = 4;
-    // above radius 5 four CTAs per multiprocessor would leave 128 registers a thread and
-    // spills (186^3: space order 12 65.9 us a step at four, 54.4 at three; 16 63.6 and 61.0)
-    static constexpr int CTAS = R <= 5 ? 4 : 3;
     static constexpr int SMEM_BYTES = S * STAGE * 4;
 };
 
@@ -78,7 +80,7 @@ struct NoallocShape {
 // 84^3 at 4 18.7 -> 10.5 us; rows of 16 / 4 bytes alignment (186 x 186 x 188 / 185 at 8)
 // 82.8 / 80.2 -> 35.1 / 46.6 us.
 template <int R, int VEC>
-__global__ void __launch_bounds__(128, NoallocShape<R>::CTAS) noalloc_step_kernel(const StepArgs a, unsigned *scratch) {
+__global__ void __launch_bounds__(128, noalloc_ctas_per_sm(R)) noalloc_step_kernel(const StepArgs a, unsigned *scratch) {
     using G = NoallocShape<R>;
     constexpr int TZ = G::TZ, TY = G::TY, SW = G::SW, SH = G::SH, RZ = G::RZ, S = G::S, W = G::W;
     constexpr int U = TmaUnroll<R, kExpanded>::U, Q = 2 * R + U, NWIN = 4 + 2 * RZ;
@@ -351,8 +353,8 @@ extern "C" int fd_forward_noalloc(float *d_u, float *d_u_prev, const float *d_m,
     if (nt < 0 || step0 < 0) return fail(FD_EINVAL, "nt and step0 must be >= 0");
     const int r = space_order / 2;
     const int tiles_z = (Nz + kTileZ - 1) / kTileZ;
-    if ((long long)tiles_z * ((Ny + 7) / 8) > kNoAllocMaxCtas)
-        return fail(FD_EINVAL, "Ny*Nz too large: one step would need more than 16384 CTAs of scratch");
+    if ((long long)tiles_z * ((Ny + 7) / 8) > kNoAllocMaxTiles)
+        return fail(FD_EINVAL, "Ny*Nz too large: a y-z plane may hold at most 16384 tiles of 8 x 32 points");
     // per-device set-up: the address of this device's copy of the scratch array
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNoAllocMaxDevices)
@@ -379,7 +381,7 @@ extern "C" int fd_forward_noalloc(float *d_u, float *d_u_prev, const float *d_m,
     // ones 100.3), but none shorter than 8 unless the domain is: a chunk also loads its 2r
     // neighbouring planes
     const long long tiles = (long long)tiles_z * ((Ny + 15) / 16);
-    const long long slots = (long long)(r <= 5 ? 4 : 3) * sms;  // NoallocShape::CTAS
+    const long long slots = (long long)noalloc_ctas_per_sm(r) * sms;
     const long long chunks = std::max<long long>(
         1, std::min<long long>(std::max<long long>(slots / tiles, (Nx + 23) / 24), Nx / 8));
     const int x_block = int((Nx + chunks - 1) / chunks);
