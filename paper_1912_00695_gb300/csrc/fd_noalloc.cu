@@ -75,10 +75,11 @@ struct NoallocShape {
 // Bound: instruction issue and latency at 12 to 16 warps per multiprocessor (the copies in
 // pieces add to the arithmetic), not memory. It replaces one point per thread with halos
 // staged through registers and a second launch per step for the maximum. Time a step,
-// before -> now (one GB300, damped, 50 steps): 186^3 at space order 2 / 8 / 12 / 16
-// 55.1 / 78.2 / 88.7 / 96.5 -> 30.5 / 39.5 / 54.7 / 63.1 us; 276^3 at 8 282 -> 97.5 us;
-// 84^3 at 4 18.7 -> 10.5 us; rows of 16 / 4 bytes alignment (186 x 186 x 188 / 185 at 8)
-// 82.8 / 80.2 -> 35.1 / 46.6 us.
+// before -> now (one GB300, a damped 10-point layer on every side, 150 steps): 186^3 at
+// space order 2 / 8 / 12 / 16 55.1 / 79.5 / 87.0 / 95.4 -> 35.4 / 45.2 / 62.1 / 70.7 us;
+// 276^3 at 8 287 -> 106 us; 84^3 at 4 18.6 -> 10.3 us; rows of 16 / 4 bytes alignment
+// (186 x 186 x 188 / 185 at 8) 80.3 / 78.4 -> 37.4 / 53.9 us. Without damping (no divisions)
+// 186^3 at 8 65.7 -> 34.9 us, 276^3 279 -> 92.3 us.
 template <int R, int VEC>
 __global__ void __launch_bounds__(128, noalloc_ctas_per_sm(R)) noalloc_step_kernel(const StepArgs a, unsigned *scratch) {
     using G = NoallocShape<R>;
@@ -376,10 +377,10 @@ extern "C" int fd_forward_noalloc(float *d_u, float *d_u_prev, const float *d_m,
         scratch = g_noalloc_ptr[dev];
         sms = g_noalloc_sms[dev];
     }
-    // x-chunks: as many as fill the resident CTA slots once, and no longer than 24 planes (at
-    // 276^3 one wave of 92-plane chunks took 114.9 us a step, 24-plane chunks 94.6, 12-plane
-    // ones 100.3), but none shorter than 8 unless the domain is: a chunk also loads its 2r
-    // neighbouring planes
+    // x-chunks: as many as fill the resident CTA slots once, and no longer than 24 planes
+    // (276^3 damped, space order 8: one wave of 92-plane chunks 124.3 us a step, this rule's 23
+    // planes 105.9, 24 planes 100.5, 12 planes 104.6), but none shorter than 8 unless the domain
+    // is: a chunk also loads its 2r neighbouring planes
     const long long tiles = (long long)tiles_z * ((Ny + 15) / 16);
     const long long slots = (long long)noalloc_ctas_per_sm(r) * sms;
     const long long chunks = std::max<long long>(
