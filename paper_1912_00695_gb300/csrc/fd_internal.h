@@ -26,11 +26,19 @@ constexpr int kModeStep = 0, kModeForwardD = 1, kModeAdjointGrad = 2;
 // at R = 8).
 constexpr int kTmaWarpsPerSM = 16;
 // Above radius 8 the register queue needs more than 128 registers per thread. Radii 9 and 10
-// factored and 9 expanded are compiled for 8 warps per SM and fit 12 by themselves; radii 11
-// and 12, and 10 expanded, are held to the 168 registers that 12 warps leave (276^3, flow,
-// held / not: space order 24 factored 188.3 / 161.2 Gpts/s, expanded 135.4 / 120.8, in BF16
-// 151.7 / 134.3, 20 expanded at 220^3 149.4 / 129.2; but 18 and 20 factored 221.1 / 235.8 and
-// 209.5 / 221.2, 18 expanded 166.2 / 171.7).
+// factored and 9 expanded are compiled for 8 warps per SM: in 32x16 tiles their flow kernels
+// take 154 to 168 registers and their per-step kernels 154 to 166, so that 12 warps fit all the
+// same; only the per-step FP32 kernel of radius 10 (172), and of the gradient's passes the
+// adjoint of radius 9 (172) and both of radius 10 (172, 180), run 8. Radii 11 and 12, and 10
+// expanded, are held to the 168 registers that 12 warps leave (276^3, flow, held / not: space
+// order 24 factored 188.3 / 161.2 Gpts/s, expanded 135.4 / 120.8, 20 expanded at 220^3 149.4 /
+// 129.2; but 18 and 20 factored 221.1 / 235.8 and 209.5 / 221.2, 18 expanded 166.2 / 171.7; the
+// gradient's two passes at 22 and 24, 200^3, 112 / 121 and 117 / 127 us a step).
+// BF16 at 22 and 24: 161.5 / 150.9 and 152.4 / 138.5 on the flow, where the plane loop with its
+// sources inline and a voting barrier had 166.4 and 153.8 unheld: these two lost 3 and 1 % to
+// the change that gave every other radius and form more (their per-step launches gained too,
+// 174 -> 141 and 184 -> 149 us a step); putting back any part of that loop for them measured
+// slower still.
 // Two y rows per thread double the x queues: 8 warps per SM.
 constexpr int tma_warps_per_sm(int r, int rows = 1, int form = 0) {
     return rows > 1 ? 8 : r <= 8 ? kTmaWarpsPerSM : r > 10 || (form != 0 && r > 9) ? 12 : 8;
