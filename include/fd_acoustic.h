@@ -275,7 +275,7 @@ int fd_forward_two_step(fd_handle *hd, int nt);
  * gives up (about 2 s) ends the launch and sets FD_ETIMEOUT in the status.
  * The x-chunk length is the options' x_block if set, else timed on the
  * first steps of the first call of at least 144 steps for the grid and launch
- * shape (candidates 8-64 planes, 8 steps each; all of them part of the
+ * shape (candidates 8-64 planes, 4-56 on small grids, 8 steps each; all of them part of the
  * requested steps, same bits) and cached for the process; a shorter first
  * call takes the multiple of 4 planes, up to 40, that gives about 1.7 items a
  * step per resident CTA (and fd_forward runs an FP32 shot's per-step launches for

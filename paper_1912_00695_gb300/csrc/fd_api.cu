@@ -1750,8 +1750,6 @@ static int flow_tables(fd_handle *hd, int xb, int nbz, int nby, int nbx) {
     return FD_OK;
 }
 
-// Flow launch arguments for nt steps from the handle's state with x-chunks of
-// xb planes; *bytes: the zeroed prefix of the flow buffer (counter, abort, flags).
 // CTAs of the handle's flow kernel that the GPU holds at a time (0: no such kernel).
 static int flow_slots(fd_handle *hd, bool ex) {
     int &flow_ctas = ex ? hd->flow_ctas_ex : hd->flow_ctas;
@@ -1763,6 +1761,8 @@ static int flow_slots(fd_handle *hd, bool ex) {
     return flow_ctas;
 }
 
+// Flow launch arguments for nt steps from the handle's state with x-chunks of
+// xb planes; *bytes: the zeroed prefix of the flow buffer (counter, abort, flags).
 static int make_flow_args(fd_handle *hd, int nt, int xb, FlowArgs *f, size_t *bytes, int *ctas) {
     const int nbz = (hd->Nz + hd->tile_z - 1) / hd->tile_z, nby = (hd->Ny + hd->tile_y - 1) / hd->tile_y;
     const int nbx = (hd->Nx + xb - 1) / xb;
@@ -2632,9 +2632,6 @@ constexpr int kBatchTuneMinShots = 4;
 constexpr int kBatchLongSteps = 9;   // the long probes of the schedule choice
 constexpr int kBatchFlowXb = 48;     // the flow's second x-chunk candidate
 
-// Times every candidate shape on kBatchTuneSteps real steps of this forward (*nt is
-// reduced by the steps they took) and keeps the fastest for the batch's lifetime.
-// Runs once, on the first forward long enough with at least kBatchTuneMinShots shots.
 // FP32 batches: whether one persistent launch per forward (the flow schedule) beats
 // one launch per step on the tuned shape. The flow is timed at the tuned x-chunks and
 // at kBatchFlowXb-plane chunks (shorter items balance a persistent launch better);

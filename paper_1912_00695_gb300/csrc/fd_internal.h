@@ -37,8 +37,8 @@ constexpr int kTmaWarpsPerSM = 16;
 // BF16 at 22 and 24: 161.5 / 150.9 and 152.4 / 138.5 on the flow, where the plane loop with its
 // sources inline and a voting barrier had 166.4 and 153.8 unheld: these two lost 3 and 1 % to
 // the change that gave every other radius and form more (their per-step launches gained too,
-// 174 -> 141 and 184 -> 149 us a step); putting back any part of that loop for them measured
-// slower still.
+// 174 -> 141 and 184 -> 149 us a step); parts of that loop put back for these two alone gave
+// +0.5 to -10 %.
 // Two y rows per thread double the x queues: 8 warps per SM.
 constexpr int tma_warps_per_sm(int r, int rows = 1, int form = 0) {
     return rows > 1 ? 8 : r <= 8 ? kTmaWarpsPerSM : r > 10 || (form != 0 && r > 9) ? 12 : 8;

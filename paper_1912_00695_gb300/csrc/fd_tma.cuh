@@ -752,7 +752,11 @@ __device__ __forceinline__ void tma_finish(TmaAcc &acc, const ScaleState &sc) {
 
 // Step kernels are launched with programmatic stream serialization: their launch is processed
 // while the stream's previous kernel ends, and each CTA, its ring set up, waits for that
-// kernel's completion before it touches device memory. us a step of the per-step launches,
+// kernel's completion before it touches a field, a scale or the status. (The batch kernel reads
+// its work items, arguments and tensor maps before the wait: the first launch of a sequence,
+// which follows their upload, does not overlap, and nothing may write those tables between the
+// steps of one sequence. A handle's step reads nothing that another stream writes, but for a
+// slab's halo: slabs do not overlap.) us a step of the per-step launches,
 // without -> with (one GB300): 84^3 at space order 4 / 8 5.4 / 6.9 -> 5.0 / 5.6, 100^3 at 16
 // 11.0 -> 9.5, 80^3 in FP16 at 4 5.7 -> 5.1, 276^3 at 8 67.7 -> 67.1. (Letting the next
 // kernel's CTAs become resident during a step, by an early trigger, gave 1 to 2 % more on some
